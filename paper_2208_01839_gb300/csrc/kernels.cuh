@@ -177,6 +177,8 @@ struct RasDev {
 };
 constexpr int32_t SOLVE_RING_FULL = 2 * SOLVE_BUF_BLOCKS_DEV;
 constexpr int32_t SOLVE_RING_HALF = SOLVE_BUF_BLOCKS_DEV;
+// contexts of at most this many subdomains (one per SM) take the solve's WIDE form
+constexpr int32_t SOLVE_WIDE_MAX = 152;
 constexpr int32_t SOLVE_WAIT_POLLS_DEFAULT = 1 << 20;
 void launch_ilu_factor(const RasDev& d, const double* val, const float* val32, int32_t* err, bool fp32,
                        cudaStream_t s);

@@ -252,24 +252,30 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int po
 // copy is in flight into the shared memory of a CTA that has left
 constexpr int SOLVE_DRAIN_POLLS = 1 << 20;
 
-// Stage data of one subdomain stream through two rings in shared memory: the
-// factor blocks (SolveRing<T>::blocks) and the per-row records (SOLVE_RING_ROWS).
-// Warp 7 is the producer: its lane 0 reads the level plan and issues the bulk
-// copies of up to SOLVE_SLOTS stages ahead, as far as both rings have room;
-// a stage's "full" mbarrier completes when its bytes have landed, and its
-// "empty" mbarrier when the consumers are done with it.  Warps 0-6 consume
-// the stages in order and meet at a named barrier after each one (the rows of
-// a level depend on the rows of earlier levels).  A stage never wraps around a
-// ring's end: the producer skips the tail.  Every wait is bounded; on a
-// timeout the kernel sets bit 3 of *err, lets every issued copy land and
-// returns.
-// Ring of factor blocks: two stages (236 blocks: 49 KB in FP64, 26 KB in FP32) so that
-// the next stage streams in while one is consumed, or one stage (118 blocks), which
-// halves a CTA's shared memory so that more subdomains share an SM and hide each
-// other's latency instead (SOLVE_RING_FULL / SOLVE_RING_HALF; a 354-block FP32 ring
-// measured 6% slower).
-constexpr int SOLVE_RING_ROWS = 2 * SOLVE_BUF_ROWS_DEV;
+// Stage data of one subdomain stream through shared memory: the factor blocks
+// (SolveRing blocks), the per-row records and the rows' first values (r in the forward
+// sweep, the forward result in the backward one; SOLVE_RING_ROWS rows).  Warp NCW is
+// the producer: its lane 0 reads the level plan and issues the bulk copies of up to
+// SOLVE_SLOTS stages ahead, as far as the rings have room, and all its lanes gather
+// the first values by cp.async; a stage's "full" mbarrier completes when all of them
+// have landed, and its "empty" mbarrier when the consumers are done with it.  The
+// consumer warps take the stages in order and meet at a named barrier after each one
+// (the rows of a level depend on the rows of earlier levels).  A stage never wraps
+// around a ring's end: the producer skips the tail.  The producer starts the backward
+// sweep's stages once the forward sweep is complete (their first values are its
+// results).  Every wait is bounded; on a timeout the kernel sets bit 3 of *err, lets
+// every issued copy land and returns.
+// Solution entries are numbered by their position in the sweep; the last SOLVE_WIN of
+// them are kept in shared memory, where nearly all of a row's dependencies lie, and
+// every entry goes to the work arrays in global memory for the rest and for the
+// backward sweep.
+// Ring of factor blocks: two stages (236 blocks) or one (118), which leaves the shared
+// memory to more resident subdomains (SOLVE_RING_FULL / SOLVE_RING_HALF).
+constexpr int SOLVE_RING_ROWS = SOLVE_BUF_ROWS_DEV;
+constexpr int SOLVE_WIN = 256;
 constexpr int SOLVE_SLOTS = 8;
+static_assert(SOLVE_WIN >= 2 * SOLVE_BUF_ROWS_DEV && (SOLVE_WIN & (SOLVE_WIN - 1)) == 0,
+              "a stage's rows must not displace the window's entries that it reads");
 
 __device__ __forceinline__ void mbar_init_count(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
@@ -277,17 +283,133 @@ __device__ __forceinline__ void mbar_init_count(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// one arrival on `bar` when every cp.async this thread has issued so far has landed (the
+// arrival is part of the barrier's count)
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void cp_async_value(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_value(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
 // named barrier 1 over the NCW consumer warps (the producer warp does not take part)
 template <int NCW>
 __device__ __forceinline__ void consumers_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(32 * NCW) : "memory");
 }
 
-// NCW consumer warps (7 or 3) and one producer warp.  Seven consumers take up to 42
-// rows of a stage in one round; three take 18, but their CTA of 128 threads needs half
-// the registers, so where shared memory allows (the FP32 rings) twice as many
-// subdomains run on an SM at once.  Every row's arithmetic is the same either way.
-template <class T, class TZ, int CH, int NCW, int RB>
+// What the consumer warps share for one stage.
+template <class T>
+struct StageView {
+  const T* B;         // the stage's factor blocks
+  const int4* inf;    // its row records
+  const double* fv;   // its first values, five 8-byte slots a row (type T in the backward sweep)
+  T* vec;             // solution entries of the sweep in global memory
+  T* win;             // the last SOLVE_WIN of them
+  int nrows, k0;      // rows, sweep position of the first
+};
+
+// One stage's rows, S lanes groups to a row: a warp takes 6 / S rows, lane = 5 (part R + row) +
+// component, and part p of a row sums its blocks p, p + S, ...  An FP64 FMA occupies a
+// warp for 64 clocks whatever its lanes and dependences, and an SM runs four such warps
+// at once, so a stage of few rows is quicker with its rows' blocks spread over more
+// warps.  S = 1 keeps two chains (blocks of even and odd number) that are added at the
+// end: the same sums in the same order as the two parts of S = 2, so either may be
+// taken for any stage.  The entries of CH blocks are loaded before any of their FMAs.
+// Measured with the gathered first values and the window: 2.0M nodes, 512 subdomains,
+// ILU(1), FP64 2.36 -> 1.93 ms a solve; 1024 x 1024, FP32 0.607 -> 0.58 ms.
+template <int S, class T, class TZ, int CH, int NCW>
+__device__ __forceinline__ void stage_rows(const StageView<T>& sv, bool fw, int warp, int lane, TZ* __restrict__ z) {
+  constexpr int BS = SolveBS<T>::v;
+  constexpr int R = 6 / S;
+  const int l5 = lane / 5, cpt = lane - 5 * l5;
+  const int part = S == 1 ? 0 : l5 / R, rw = l5 - part * R;
+  const int lo = sv.k0 + sv.nrows - SOLVE_WIN;  // first position that this stage's results leave in the window
+  const int jb = fw ? 0 : 1;                    // block 0 of a backward row is the inverted pivot
+  for (int qb = warp * R; qb < sv.nrows; qb += R * NCW) {
+    const int q = qb + rw;
+    const bool act = lane < 30 && q < sv.nrows;
+    int st = 0, cn = 0, onode = -1;
+    T acc = T(0), acc2 = T(0);
+    if (act) {
+      const int4 rec = sv.inf[q];
+      st = rec.y;
+      cn = rec.z;
+      onode = rec.w;
+      if (part == 0) acc = fw ? (T)sv.fv[5 * q + cpt] : reinterpret_cast<const T*>(sv.fv + 5 * q)[cpt];
+    }
+    for (int j = jb + part; j < cn; j += S * CH) {
+      const int nb = S == 1 ? min(CH, cn - j) : min(CH, (cn - j + S - 1) / S);
+      T xv[CH][5];
+#pragma unroll
+      for (int u = 0; u < CH; ++u) {  // a short row reloads its last block to fill the batch
+        const int pos = col_of(sv.B[(st + j + S * min(u, nb - 1)) * BS + 25]);
+        const T* vk = pos >= lo ? sv.win + 5 * (pos & (SOLVE_WIN - 1)) : sv.vec + 5 * (int64_t)pos;
+#pragma unroll
+        for (int mm = 0; mm < 5; ++mm) xv[u][mm] = vk[mm];
+      }
+#pragma unroll
+      for (int u = 0; u < CH; ++u) {
+        if (u < nb) {
+          const T* Lb = sv.B + (st + j + S * u) * BS + 5 * cpt;
+#pragma unroll
+          for (int mm = 0; mm < 5; ++mm) {
+            if (S == 1 && (u & 1)) acc2 = fmaT(-Lb[mm], xv[u][mm], acc2);
+            else acc = fmaT(-Lb[mm], xv[u][mm], acc);
+          }
+        }
+      }
+      if (S == 1 && CH % 2 == 1) {  // the next batch starts on the other chain
+        const T t = acc;
+        acc = acc2;
+        acc2 = t;
+      }
+    }
+    // the parts' sums; FP addition commutes, so whichever register holds which chain of S = 1
+    // the sum is the same
+    if (S == 1) {
+      acc += acc2;
+    } else {
+      T oth[S];
+#pragma unroll
+      for (int p = 1; p < S; ++p) oth[p] = __shfl_sync(FULL, acc, (lane + 5 * R * p) & 31);
+      if (S == 2) {
+        acc += oth[1];
+      } else if (S == 3) {
+        acc += oth[1] + oth[2];
+      } else {
+#pragma unroll
+        for (int p = 1; p + 1 < S; p += 2) oth[p] += oth[p + 1];
+        if (S == 6) acc = (acc + oth[S - 1]) + (oth[1] + oth[3]);
+      }
+    }
+    const int kq = sv.k0 + q;  // this row's position
+    T v = acc;
+    if (!fw) {
+      // z = U_kk^{-1} (...): the five partial results of the row sit in lanes 5 rw .. 5 rw + 4
+      v = T(0);
+      const T* Dv = sv.B + st * BS + 5 * cpt;
+#pragma unroll
+      for (int mm = 0; mm < 5; ++mm) {
+        const T am = __shfl_sync(FULL, acc, 5 * rw + mm);
+        if (act) v = fmaT(Dv[mm], am, v);
+      }
+    }
+    if (act && part == 0) {
+      sv.vec[5 * (int64_t)kq + cpt] = v;
+      sv.win[5 * (kq & (SOLVE_WIN - 1)) + cpt] = v;
+      if (!fw && onode >= 0) z[5 * (int64_t)onode + cpt] = (TZ)v;
+    }
+  }
+}
+
+// NCW consumer warps (7 or 3) and one producer warp.  Every row's arithmetic is the same
+// for either count.  WIDE (contexts whose subdomains do not fill the SMs) splits the rows
+// of small stages over up to six parts: what counts there is a stage's own latency, and
+// nothing else uses the FP64 pipe.
+template <class T, class TZ, int CH, int NCW, int RB, bool WIDE>
 __global__ void __launch_bounds__(32 * (NCW + 1), NCW <= 3 ? 7 : 4)
     k_ilu_solve(RasDev d, const double* __restrict__ r, TZ* __restrict__ z, int32_t* err) {
   constexpr int BS = SolveBS<T>::v;
@@ -297,10 +419,12 @@ __global__ void __launch_bounds__(32 * (NCW + 1), NCW <= 3 ? 7 : 4)
   __shared__ __align__(8) uint64_t full[NS];
   __shared__ __align__(8) uint64_t empty[NS];
   __shared__ __align__(16) int4 info[RR];
-  __shared__ int slot_vb[NS], slot_vr[NS], slot_n[NS];  // virtual ring starts and row count of a stage
-  __shared__ int slot_k0[NS];                            // sweep position of a stage's first row
+  __shared__ __align__(16) int4 slot[NS];  // ring starts (blocks, rows), row count and first position of a stage
+  __shared__ int2 virt[NS];  // virtual ring starts of the stages in flight (producer's lane 0)
   __shared__ int abort_at;  // first stage at which a consumer warp's wait gave up (INT_MAX: none)
   T* ring = reinterpret_cast<T*>(smem_raw);
+  double* fv = reinterpret_cast<double*>(ring + (size_t)RB * BS);
+  T* win = reinterpret_cast<T*>(fv + 5 * RR);
   const int p = d.sd_sched ? d.sd_sched[blockIdx.x] : (int)blockIdx.x;
   const int32_t r0 = d.sd_row0[p];
   T* y = ywk<T>(d) + 5 * (int64_t)r0;
@@ -311,7 +435,7 @@ __global__ void __launch_bounds__(32 * (NCW + 1), NCW <= 3 ? 7 : 4)
   const int nstage = nF + nB;
   if (tid == 0) {
     for (int k = 0; k < NS; ++k) {
-      mbar_init_count(&full[k], 1);
+      mbar_init_count(&full[k], 33);  // lane 0's bulk copies and the 32 lanes' gathers
       mbar_init_count(&empty[k], 1);
     }
     abort_at = INT_MAX;
@@ -322,150 +446,122 @@ __global__ void __launch_bounds__(32 * (NCW + 1), NCW <= 3 ? 7 : 4)
   if (warp == NCW) {
     // ---- producer: stage g < nF is forward level g, otherwise backward level
     // g - nF; it uses slot g % NS, whose barriers complete phase (g / NS) & 1 for it.
-    if (lane != 0) return;
-    const T* fL = solve_fwd<T>(d);
-    const T* bU = solve_bwd<T>(d);
+    // The plan entries and the rows' gather indices of a stage are read one stage ahead.
+    constexpr int NU = (SOLVE_BUF_ROWS_DEV + 31) / 32;
+    int q0 = 0, nr = 0, nb = 0, id[NU];
+    int64_t b0 = 0;
+    auto plan = [&](int g, int& pq0, int& pnr, int64_t& pb0, int& pnb, int (&pid)[NU]) {
+      if (g >= nstage) return;
+      const bool fw = g < nF;
+      const SolvePlanDev& P = fw ? d.fwd : d.bwd;
+      const int32_t lv = fw ? LF + g : LB + g - nF;
+      pq0 = P.levpos[lv];
+      pnr = P.levpos[lv + 1] - pq0;
+      pb0 = P.levblk[lv];
+      pnb = (int)(P.levblk[lv + 1] - pb0);
+#pragma unroll
+      for (int u = 0; u < NU; ++u)
+        if (lane + 32 * u < pnr) pid[u] = P.info[(int64_t)r0 + pq0 + lane + 32 * u].x;
+    };
+    plan(0, q0, nr, b0, nb, id);
     int vb = 0, vr = 0, oldest = 0;  // ring heads (virtual, growing); oldest stage not known to be released
     int gi = 0;
     bool ok = true;
-    for (; gi < nstage && ok; ++gi) {
+    for (; gi < nstage; ++gi) {
       const bool fw = gi < nF;
-      const SolvePlanDev& P = fw ? d.fwd : d.bwd;
-      const int32_t lv = fw ? LF + gi : LB + gi - nF;
-      const int32_t q0 = P.levpos[lv], q1 = P.levpos[lv + 1];
-      const int64_t b0 = P.levblk[lv];
-      const int nb = (int)(P.levblk[lv + 1] - b0), nr = q1 - q0;
+      int nq0 = 0, nnr = 0, nnb = 0, nid[NU];
+      int64_t nb0 = 0;
+      plan(gi + 1, nq0, nnr, nb0, nnb, nid);
       int sb = vb, sr = vr;
       if (sb % RB + nb > RB) sb += RB - sb % RB;
       if (sr % RR + nr > RR) sr += RR - sr % RR;
-      // release stages (in order) until this one fits and its slot is free
-      while (oldest < gi &&
-             (gi - oldest >= NS || sb + nb - slot_vb[oldest % NS] > RB || sr + nr - slot_vr[oldest % NS] > RR)) {
-        if (!mbar_wait(&empty[oldest % NS], (uint32_t)((oldest / NS) & 1), d.wait_polls) ||
-            *(volatile int*)&abort_at != INT_MAX) {
-          ok = false;
-          break;
-        }
-        ++oldest;
-      }
-      if (!ok) break;
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       const int sl = gi % NS;
-      slot_vb[sl] = sb;
-      slot_vr[sl] = sr;
-      slot_n[sl] = nr;
-      slot_k0[sl] = q0;
-      const uint32_t bytes_b = (uint32_t)nb * BS * (uint32_t)sizeof(T);
-      const uint32_t bytes_i = (uint32_t)nr * (uint32_t)sizeof(int4);
-      mbar_arrive_tx(&full[sl], bytes_b + bytes_i);  // releases the slot fields above to the consumers
-      if (bytes_b) bulk_g2s(ring + (size_t)(sb % RB) * BS, (fw ? fL : bU) + b0 * BS, bytes_b, &full[sl]);
-      if (bytes_i) bulk_g2s(info + sr % RR, P.info + r0 + q0, bytes_i, &full[sl]);
+      if (lane == 0) {
+        // release stages (in order) until this one fits and its slot is free; all of the
+        // forward sweep before the first backward stage
+        while (oldest < gi) {
+          const int os = oldest % NS;
+          const int2 at = virt[os];
+          if (!(gi == nF || gi - oldest >= NS || sb + nb - at.x > RB || sr + nr - at.y > RR)) break;
+          if (!mbar_wait(&empty[os], (uint32_t)((oldest / NS) & 1), d.wait_polls) ||
+              *(volatile int*)&abort_at != INT_MAX) {
+            ok = false;
+            break;
+          }
+          ++oldest;
+        }
+      }
+      ok = __shfl_sync(FULL, (int)ok, 0) != 0;
+      if (!ok) break;
+      const int rb = sb % RB, rr = sr % RR;
+      if (lane == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        virt[sl] = make_int2(sb, sr);
+        slot[sl] = make_int4(rb, rr, nr, q0);
+        const uint32_t bytes_b = (uint32_t)nb * BS * (uint32_t)sizeof(T);
+        const uint32_t bytes_i = (uint32_t)nr * (uint32_t)sizeof(int4);
+        mbar_arrive_tx(&full[sl], bytes_b + bytes_i);  // releases the slot fields above to the consumers
+        if (bytes_b) bulk_g2s(ring + (size_t)rb * BS, (fw ? solve_fwd<T>(d) : solve_bwd<T>(d)) + b0 * BS, bytes_b, &full[sl]);
+        if (bytes_i) bulk_g2s(info + rr, (fw ? d.fwd : d.bwd).info + r0 + q0, bytes_i, &full[sl]);
+      }
+#pragma unroll
+      for (int u = 0; u < NU; ++u) {
+        const int q = lane + 32 * u;
+        if (q < nr) {
+          double* dst = fv + 5 * (rr + q);
+          if (fw) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) cp_async_value(dst + c, r + 5 * (int64_t)id[u] + c);
+          } else {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) cp_async_value(reinterpret_cast<T*>(dst) + c, y + 5 * (int64_t)id[u] + c);
+          }
+        }
+      }
+      cp_async_arrive(&full[sl]);
       vb = sb + nb;
       vr = sr + nr;
+      q0 = nq0;
+      nr = nnr;
+      b0 = nb0;
+      nb = nnb;
+#pragma unroll
+      for (int u = 0; u < NU; ++u) id[u] = nid[u];
     }
-    if (!ok) atomicOr(err, 8);
+    if (!ok && lane == 0) atomicOr(err, 8);
     // every issued copy lands before the CTA can exit (the last stage issued on
     // each slot is the only one whose phase is still open)
-    for (int k = gi - 1; k >= 0 && k >= gi - NS; --k)
-      mbar_wait(&full[k % NS], (uint32_t)((k / NS) & 1), SOLVE_DRAIN_POLLS);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (lane == 0)
+      for (int k = gi - 1; k >= 0 && k >= gi - NS; --k)
+        mbar_wait(&full[k % NS], (uint32_t)((k / NS) & 1), SOLVE_DRAIN_POLLS);
     return;
   }
 
-  // ---- consumers (warps 0-6)
-  // Solution entries are numbered by their position in the sweep: y (forward) and
-  // z (backward) of position k live at 5 k in the subdomain's work arrays, so a
-  // stage writes one contiguous run and reads the runs of earlier stages.  (A
-  // shared-memory window of recent entries measured slower: the dependency loads
-  // hit L1, and the window's shared memory comes out of L1.)
-  const int rw = lane / 5, cpt = lane - 5 * rw;
+  // ---- consumers (warps 0 .. NCW - 1)
   // A warp whose wait gives up skips the stage and records it; every consumer
   // reads abort_at after the named barrier that closes the stage, and only
   // values <= g (written before that barrier) end the loop at stage g, so all
   // consumer warps leave at the same stage.
   bool aborted = false;
+  StageView<T> sv;
+  sv.win = win;
   for (int g = 0; g < nstage; ++g) {
     const bool fw = g < nF;
     const int sl = g % NS;
     const bool landed = __all_sync(FULL, mbar_wait(&full[sl], (uint32_t)((g / NS) & 1), d.wait_polls));
     if (!landed && lane == 0) atomicMin(&abort_at, g);
-    const T* B = ring + (size_t)(slot_vb[sl] % RB) * BS;
-    const int4* inf = info + slot_vr[sl] % RR;
-    const int nrows = landed ? slot_n[sl] : 0;
-    const int k0 = slot_k0[sl];
-    T* vec = fw ? y : zz;
-    for (int qb = warp * 6; qb < nrows; qb += 6 * NCW) {
-      const int q = qb + rw;
-      const bool act = lane < 30 && q < nrows;
-      int32_t st = 0, cn = 0, onode = -1;
-      T acc = T(0), acc2 = T(0);
-      if (act) {
-        const int4 rec = inf[q];
-        st = rec.y;
-        cn = rec.z;
-        onode = rec.w;
-        // forward: r of the row's node; backward: the row's forward result
-        acc = fw ? (T)r[5 * (int64_t)rec.x + cpt] : y[5 * rec.x + cpt];
-      }
-      // y_k -= sum L y_j (forward) or y_k - sum U z_j (backward, block 0 is the
-      // inverted pivot).  The entries of CH blocks are loaded before any of their
-      // FMAs, so a row waits for one memory latency per CH blocks, not per block.
-      // A short row reloads its last block to fill the batch; a stage is bound by
-      // its busiest warp's instruction chain, so the batch trades load rounds
-      // against instructions (2.0M nodes: FP32 0.91 ms for 2 blocks against 0.96 /
-      // 0.95 / 0.94 / 1.02 ms for 1 / 4 / 3 / 6; FP64 1.68 ms against 1.74 / 1.70 ms
-      // for 1 / 3); the autotuner picks CH per context.  Block b of the row (counted
-      // from its first product) goes to chain b % 2 whatever CH is: both chains
-      // subtract, the slot of a batch's block u is fixed (u % 2), and after a batch
-      // of odd size the two chains trade slots, so every CH gives the same sums in
-      // the same order with no run-time choice of chain per FMA.
-      const int32_t jb = fw ? 0 : 1;
-      for (int32_t j = jb; j < cn; j += CH) {
-        const int nb = min(CH, cn - j);
-        T xv[CH][5];
-#pragma unroll
-        for (int u = 0; u < CH; ++u) {
-          const T* vk = vec + 5 * (int64_t)col_of(B[(st + j + min(u, nb - 1)) * BS + 25]);
-#pragma unroll
-          for (int mm = 0; mm < 5; ++mm) xv[u][mm] = vk[mm];
-        }
-#pragma unroll
-        for (int u = 0; u < CH; ++u) {
-          if (u < nb) {  // folded into two accumulator chains: no separate add per block
-            const T* Lb = B + (st + j + u) * BS + 5 * cpt;
-#pragma unroll
-            for (int mm = 0; mm < 5; ++mm) {
-              if (u & 1) acc2 = fmaT(-Lb[mm], xv[u][mm], acc2);
-              else acc = fmaT(-Lb[mm], xv[u][mm], acc);
-            }
-          }
-        }
-        if (CH % 2 == 1) {  // the next batch starts on the other chain
-          const T t = acc;
-          acc = acc2;
-          acc2 = t;
-        }
-      }
-      // the chain that started from r (or y) and the other one; FP addition commutes, so
-      // whichever register holds which chain the sum is the same (and -fma(a, b, c) =
-      // fma(-a, b, -c) exactly, so this equals the r - sum_even - (sum_odd) of a chain that adds)
-      acc += acc2;
-      const int kq = k0 + q;  // this row's position
-      T v = acc;
-      if (!fw) {
-        // z = U_kk^{-1} (...): the five partial results of the row sit in lanes 5 rw .. 5 rw + 4
-        v = T(0);
-        const T* Dv = B + st * BS + 5 * cpt;
-#pragma unroll
-        for (int mm = 0; mm < 5; ++mm) {
-          const T am = __shfl_sync(FULL, acc, 5 * rw + mm);
-          if (act) v = fmaT(Dv[mm], am, v);
-        }
-      }
-      if (act) {
-        vec[5 * (int64_t)kq + cpt] = v;
-        if (!fw && onode >= 0) z[5 * (int64_t)onode + cpt] = (TZ)v;
-      }
-    }
+    const int4 ds = slot[sl];
+    sv.B = ring + (size_t)ds.x * BS;
+    sv.inf = info + ds.y;
+    sv.fv = fv + 5 * ds.y;
+    sv.vec = fw ? y : zz;
+    sv.nrows = landed ? ds.z : 0;
+    sv.k0 = ds.w;
+    if (WIDE && sv.nrows <= 7) stage_rows<6, T, TZ, CH, NCW>(sv, fw, warp, lane, z);
+    else if (WIDE && sv.nrows <= 14) stage_rows<3, T, TZ, CH, NCW>(sv, fw, warp, lane, z);
+    else if (sv.nrows <= 3 * NCW) stage_rows<2, T, TZ, CH, NCW>(sv, fw, warp, lane, z);
+    else stage_rows<1, T, TZ, CH, NCW>(sv, fw, warp, lane, z);
     consumers_sync<NCW>();  // every row of this stage is written; the stage's ring space is free
     if (*(volatile int*)&abort_at <= g) {
       aborted = true;
@@ -720,9 +816,10 @@ void launch_ilu_factor(const RasDev& d, const double* val, const float* val32, i
   count_launch();
 }
 
-size_t solve_smem(bool fp32, int ring_blocks) {
-  return fp32 ? (size_t)ring_blocks * SolveBS<float>::v * sizeof(float)
-              : (size_t)ring_blocks * SolveBS<double>::v * sizeof(double);
+// dynamic shared memory of a solve CTA: factor ring, first values, solution window
+template <class T>
+constexpr size_t solve_smem(int ring_blocks) {
+  return ((size_t)ring_blocks * SolveBS<T>::v + 5 * SOLVE_WIN) * sizeof(T) + 5 * SOLVE_RING_ROWS * sizeof(double);
 }
 
 void launch_ilu_reorg(const RasDev& d, int64_t nfwd, int64_t nbwd, const int64_t* fsrc, const int32_t* fcol,
@@ -741,14 +838,14 @@ void launch_ilu_reorg(const RasDev& d, int64_t nfwd, int64_t nbwd, const int64_t
 
 // CTAs of one solve variant that the GPU holds at once (SMs x resident CTAs per SM), found
 // once per variant; 0 if the occupancy query fails (the launch order is then always used)
-template <class T, int CH, int NCW, int RB>
-int solve_slots(size_t sm) {
-  static const int slots = [sm] {
+template <class T, int CH, int NCW, int RB, bool WIDE>
+int solve_slots() {
+  static const int slots = [] {
     int dev = 0, nsm = 0, nb = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ilu_solve<T, T, CH, NCW, RB>, 32 * (NCW + 1), sm) !=
-            cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ilu_solve<T, T, CH, NCW, RB, WIDE>, 32 * (NCW + 1),
+                                                      solve_smem<T>(RB)) != cudaSuccess) {
       (void)cudaGetLastError();  // the query's own error: nothing was launched
       return 0;
     }
@@ -761,35 +858,42 @@ int solve_slots(size_t sm) {
 // (18.4M nodes, 4096 subdomains: 7.5% off the solve).  When every CTA is resident from
 // the start it only decides which CTAs share an SM, and the natural order measured
 // slightly better (2.0M nodes, 512 subdomains: 2.5%), so a single wave keeps it.
-template <class T, int CH, int NCW, int RB>
+template <class T, int CH, int NCW, int RB, bool WIDE>
 void launch_ilu_solve_c(const RasDev& d, const double* r, T* z, int32_t* err, cudaStream_t s) {
-  const size_t sm = solve_smem(sizeof(T) == 4, RB);
   RasDev dl = d;
-  if (d.P <= solve_slots<T, CH, NCW, RB>(sm)) dl.sd_sched = nullptr;
-  k_ilu_solve<T, T, CH, NCW, RB><<<d.P, 32 * (NCW + 1), sm, s>>>(dl, r, z, err);
+  if (d.P <= solve_slots<T, CH, NCW, RB, WIDE>()) dl.sd_sched = nullptr;
+  k_ilu_solve<T, T, CH, NCW, RB, WIDE><<<d.P, 32 * (NCW + 1), solve_smem<T>(RB), s>>>(dl, r, z, err);
 }
 
-template <class T, int NCW, int RB>
-void launch_ilu_solve_w(const RasDev& d, const double* r, T* z, int32_t* err, cudaStream_t s, int ch) {
-  switch (ch) {
-    case 1: launch_ilu_solve_c<T, 1, NCW, RB>(d, r, z, err, s); break;
-    case 3: launch_ilu_solve_c<T, 3, NCW, RB>(d, r, z, err, s); break;
-    case 4: launch_ilu_solve_c<T, 4, NCW, RB>(d, r, z, err, s); break;
-    default: launch_ilu_solve_c<T, 2, NCW, RB>(d, r, z, err, s); break;
-  }
-  count_launch();
+// f.template operator()<CH, NCW, RB, WIDE>() for the launch shape of d
+template <class F>
+void solve_variant(const RasDev& d, F&& f) {
+  auto ring = [&]<int CH, int NCW, bool WIDE>() {
+    if (d.solve_ring == SOLVE_RING_HALF) f.template operator()<CH, NCW, SOLVE_RING_HALF, WIDE>();
+    else f.template operator()<CH, NCW, SOLVE_RING_FULL, WIDE>();
+  };
+  auto warps = [&]<int CH, bool WIDE>() {
+    if (d.solve_warps == 3) ring.template operator()<CH, 3, WIDE>();
+    else ring.template operator()<CH, 7, WIDE>();
+  };
+  auto batch = [&]<bool WIDE>() {
+    switch (d.solve_ch) {
+      case 1: warps.template operator()<1, WIDE>(); break;
+      case 3: warps.template operator()<3, WIDE>(); break;
+      case 4: warps.template operator()<4, WIDE>(); break;
+      default: warps.template operator()<2, WIDE>(); break;
+    }
+  };
+  if (d.P <= SOLVE_WIDE_MAX) batch.template operator()<true>();
+  else batch.template operator()<false>();
 }
 
 template <class T>
 void launch_ilu_solve_t(const RasDev& d, const double* r, T* z, int32_t* err, cudaStream_t s) {
-  const bool half = d.solve_ring == SOLVE_RING_HALF;
-  if (d.solve_warps == 3) {
-    if (half) launch_ilu_solve_w<T, 3, SOLVE_RING_HALF>(d, r, z, err, s, d.solve_ch);
-    else launch_ilu_solve_w<T, 3, SOLVE_RING_FULL>(d, r, z, err, s, d.solve_ch);
-  } else {
-    if (half) launch_ilu_solve_w<T, 7, SOLVE_RING_HALF>(d, r, z, err, s, d.solve_ch);
-    else launch_ilu_solve_w<T, 7, SOLVE_RING_FULL>(d, r, z, err, s, d.solve_ch);
-  }
+  solve_variant(d, [&]<int CH, int NCW, int RB, bool WIDE>() {
+    launch_ilu_solve_c<T, CH, NCW, RB, WIDE>(d, r, z, err, s);
+  });
+  count_launch();
 }
 
 void launch_ilu_solve(const RasDev& d, const double* r, double* z, int32_t* err, cudaStream_t s) {
@@ -800,25 +904,25 @@ void launch_ilu_solve32(const RasDev& d, const double* r, float* z, int32_t* err
   launch_ilu_solve_t<float>(d, r, z, err, s);
 }
 
-template <class T, int NCW, int RB>
-void solve_attrs() {
-  const int smem = (int)solve_smem(sizeof(T) == 4, RB);
-  cudaFuncSetAttribute(k_ilu_solve<T, T, 1, NCW, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_ilu_solve<T, T, 2, NCW, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_ilu_solve<T, T, 3, NCW, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_ilu_solve<T, T, 4, NCW, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  // the resident-CTA counts, found here (at context creation) rather than in a captured launch
-  (void)solve_slots<T, 1, NCW, RB>(smem);
-  (void)solve_slots<T, 2, NCW, RB>(smem);
-  (void)solve_slots<T, 3, NCW, RB>(smem);
-  (void)solve_slots<T, 4, NCW, RB>(smem);
-}
+// shared-memory limits and resident-CTA counts of every solve variant, set and found here (at
+// context creation) rather than in a captured launch
 template <class T>
 void solve_attrs_all() {
-  solve_attrs<T, 7, SOLVE_RING_FULL>();
-  solve_attrs<T, 3, SOLVE_RING_FULL>();
-  solve_attrs<T, 7, SOLVE_RING_HALF>();
-  solve_attrs<T, 3, SOLVE_RING_HALF>();
+  RasDev d{};
+  for (int P : {1, SOLVE_WIDE_MAX + 1})
+    for (int w : {3, 7})
+      for (int rb : {SOLVE_RING_HALF, SOLVE_RING_FULL})
+        for (int ch : {1, 2, 3, 4}) {
+          d.P = P;
+          d.solve_warps = w;
+          d.solve_ring = rb;
+          d.solve_ch = ch;
+          solve_variant(d, []<int CH, int NCW, int RB, bool WIDE>() {
+            cudaFuncSetAttribute(k_ilu_solve<T, T, CH, NCW, RB, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)solve_smem<T>(RB));
+            (void)solve_slots<T, CH, NCW, RB, WIDE>();
+          });
+        }
 }
 
 void launch_coarse_assemble(const CoarseDev& c, const double* val, const float* val32, cudaStream_t s) {
