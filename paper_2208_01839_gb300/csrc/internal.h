@@ -71,25 +71,26 @@ struct HostSetup {
   std::vector<int32_t> bwd_order, bwd_lev, sd_bwd_lev0;
   int32_t max_levels = 0;
   int32_t max_sd_rows = 0;
+  bool fp32 = false;                // FP32 subdomain factors (options.precision = 1): the solve's ring sizes
   int32_t ilu_fill = 0;             // levels of fill of the subdomain factors (options.ilu_fill)
-  // ILU(0) solve plans: the solve reads factor blocks from a copy laid out in
-  // level order (forward: each row's strictly lower blocks; backward: each row's
-  // inverted pivot block, then its upper blocks), so that every level is one
-  // contiguous range that is prefetched into shared memory while the previous
-  // level computes.  Levels are split so that a range fits the buffer.
+  // ILU solve plans: the solve reads factor blocks from a copy laid out in level order
+  // (forward: each row's inverted pivot block, then its strictly lower blocks; backward:
+  // its strictly upper blocks), so that every level is one contiguous range that is
+  // prefetched into shared memory while the previous level computes.  Levels are split so
+  // that a range fits the buffer.
   struct SolvePlan {
-    std::vector<int32_t> row;     // [NL] local row at each position (per subdomain, level order)
-    std::vector<int64_t> start;   // [NL] first block (absolute, in the solve copy) of each position
-    std::vector<int32_t> cnt;     // [NL] blocks of each position
     std::vector<int32_t> levpos;  // per subdomain nlev+1 entries: position boundaries (relative)
     std::vector<int64_t> levblk;  // per subdomain nlev+1 entries: block boundaries (absolute)
-    std::vector<int32_t> sd_lev0; // [P+1] offsets into levpos/levblk
+    std::vector<int4> stage;      // per levpos entry: the stage's record (stage_rows and the like in kernels.cuh)
+    std::vector<int32_t> sd_lev0; // [P+1] offsets into levpos/levblk/stage
     std::vector<int64_t> src;     // [nblocks] factor block (>= 0) or -1-R for the inverted pivot of row R
-    std::vector<int32_t> col;     // [nblocks] sweep position of the entry each block multiplies (own for a pivot)
-    std::vector<int32_t> info;    // [NL][4] per position: forward (node, first block in its stage, blocks, 0),
-                                  // backward (forward position, first block, blocks, node if owned else -1)
-    int32_t max_lev_blocks = 0;
+    std::vector<int32_t> col;     // [nblocks] sweep position of the entry each block multiplies, -1 - position for an
+                                  // entry that has left the window; pivots (0) multiply the row's own first value
+    std::vector<int32_t> brow;    // [nblocks] row R (absolute) of each block
+    std::vector<int32_t> info;    // [NL][4] per position: forward (node, first block in its stage, blocks, backward
+                                  // position), backward (forward position, first block, blocks, node if owned else -1)
   } sp_fwd, sp_bwd;
+  int64_t max_row_blocks = 0;  // longest row of either triangle, the diagonal counted with the upper one
   // launch order of the per-subdomain kernels (factor and solve): subdomains by
   // descending solve work (blocks + SOLVE_STAGE_WEIGHT x stages, both sweeps), ties in
   // index order, so the longest start first and the grid's tail holds the short ones
@@ -236,14 +237,11 @@ struct seird_ctx {
   float* ywork32 = nullptr;  // mixed-precision path
   float* zwork32 = nullptr;
   struct PlanPtrs {
-    int32_t* row = nullptr;
-    int64_t* start = nullptr;
-    int32_t* cnt = nullptr;
-    int32_t* levpos = nullptr;
-    int64_t* levblk = nullptr;
+    int4* stage = nullptr;
     int32_t* sd_lev0 = nullptr;
     int64_t* src = nullptr;
     int32_t* col = nullptr;
+    int32_t* brow = nullptr;
     int32_t* info = nullptr;
   } pf, pb;  // forward / backward solve plans
   double* fL = nullptr;  // level-ordered factor copies (FP64 path)
@@ -254,6 +252,7 @@ struct seird_ctx {
   double* pct = nullptr;     // [5n] residual between the steps of the multiplicative two-grid
   double* pcu = nullptr;     // [5n] FP64 post-smoothing correction
   float* pcu32 = nullptr;    // [5n] FP32 post-smoothing correction
+  float* pcr32 = nullptr;    // [8n] FP32 right-hand side of the mixed path's subdomain solves (padded rows)
   // coarse
   int32_t* cpos = nullptr;
   int32_t* cseg_blk = nullptr;
@@ -272,9 +271,9 @@ struct seird_ctx {
   double abytes[SEIRD_K_COUNT] = {};
   // launch shapes (options.autotune)
   int spmv_tb = 256, cgs_tile = 0, sms = 1;
-  int ilu_ch = 2;     // dependency-load batch of the subdomain solves (options.autotune)
-  int ilu_warps = 7;  // their consumer warps per CTA (7 or 3)
-  int ilu_ring = seird::SOLVE_RING_FULL;  // and factor-ring blocks (two stages or one)
+  int ilu_ch = 2;     // seird_set_launch_shapes' ilu_batch: recorded, the solves no longer batch their loads
+  int ilu_warps = 7;  // shape of the subdomain solves' CTAs (7 or 3, options.autotune)
+  int ilu_ring = seird::SOLVE_RING_FULL;  // and their factor ring (several stages or one)
   bool tuned = false;
   double* tune_buf = nullptr;
   // GMRES restart cycle captured into a CUDA graph (options.graph)

@@ -124,16 +124,54 @@ void launch_bsr_transpose(int64_t nnzb, const int32_t* tpos, const double* val, 
 
 // RAS and coarse space
 constexpr int SOLVE_BUF_BLOCKS_DEV = 118;  // factor blocks per ILU-solve stage buffer
-constexpr int SOLVE_BUF_ROWS_DEV = 128;    // rows per ILU-solve stage
+constexpr int SOLVE_BUF_ROWS_DEV = 64;     // rows per ILU-solve stage
+constexpr int SOLVE_WIN = 256;             // results of a sweep that a solve CTA keeps in shared memory
+static_assert(SOLVE_WIN >= 2 * SOLVE_BUF_ROWS_DEV && (SOLVE_WIN & (SOLVE_WIN - 1)) == 0,
+              "a stage's rows must not displace the entries that it reads");
+// Blocks of the solve's factor ring.  SOLVE_RING_FULL and SOLVE_RING_HALF name the two launch
+// shapes (several stages, or one).  The first takes the largest of these rings that leaves
+// room in an SM's shared memory for as many CTAs as the context's subdomains come to on 152
+// SMs: a stage's blocks then arrive several stages ahead.
+constexpr int32_t SOLVE_RING_FULL = 2 * SOLVE_BUF_BLOCKS_DEV;
+constexpr int32_t SOLVE_RING_HALF = SOLVE_BUF_BLOCKS_DEV;
+constexpr int32_t SOLVE_RING_1 = 640;    // one CTA per SM
+constexpr int32_t SOLVE_RING_2 = 400;    // FP64, two CTAs per SM; FP32, three
+constexpr int32_t SOLVE_RING_3 = 268;    // FP64, three
+constexpr int32_t SOLVE_RING_4 = 188;    // FP64, four
+constexpr int32_t SOLVE_RING_4F = 354;   // FP32, four
+// rows of the record and first-value rings that go with a block ring
+__host__ __device__ constexpr int32_t solve_ring_rows(int32_t blocks) {
+  return blocks >= SOLVE_RING_1 ? 256 : blocks >= SOLVE_RING_2 ? 160 : blocks >= SOLVE_RING_FULL ? 96 : 64;
+}
+// contexts of at most this many subdomains (one per SM) take the solve's WIDE form
+constexpr int32_t SOLVE_WIDE_MAX = 152;
+// (max_row: the longest row, HostSetup::max_row_blocks)
+inline int32_t solve_ring_blocks(int64_t P, bool fp32, bool half, int64_t max_row) {
+  if (half) return SOLVE_RING_HALF;
+  if (P <= SOLVE_WIDE_MAX) return SOLVE_RING_1;
+  const int64_t per_sm = (P + 151) / 152;
+  if (fp32) return per_sm <= 3 ? SOLVE_RING_2 : per_sm == 4 ? SOLVE_RING_4F : SOLVE_RING_FULL;
+  return per_sm <= 2 ? SOLVE_RING_2 : per_sm == 3 || max_row > SOLVE_RING_4 ? SOLVE_RING_3 : SOLVE_RING_4;
+}
+constexpr int SOLVE_RING_SPARE = 2;        // ring blocks beyond SOLVE_RING_*: a longest row with its inverted pivot
+constexpr int SOLVE_SLOTS = 16;            // stages in flight
+constexpr int SOLVE_FREE = 63;             // distance of a stage that no earlier one is in the way of
+// A stage's record: first position; first block; rows, blocks << 8 and its offset in the row
+// ring << 16 + 8 v; its offset in the block ring << 16 v and the distance back to the last
+// stage in its way << 10 + 16 v (v = 0: the longer ring, 1: SOLVE_RING_HALF).
+__host__ __device__ inline int stage_rows(int4 s) { return s.z & 255; }
+__host__ __device__ inline int stage_blocks(int4 s) { return (s.z >> 8) & 255; }
+__host__ __device__ inline int stage_row_offset(int4 s, int v) { return (s.z >> (16 + 8 * v)) & 255; }
+__host__ __device__ inline int stage_block_offset(int4 s, int v) { return (s.w >> (16 * v)) & 1023; }
+__host__ __device__ inline int stage_distance(int4 s, int v) { return (s.w >> (10 + 16 * v)) & 63; }
 struct SolvePlanDev {
-  const int32_t* row;
-  const int64_t* start;
-  const int32_t* cnt;
-  const int32_t* levpos;
-  const int64_t* levblk;
-  const int32_t* sd_lev0;
-  const int4* info;  // per position: row, first block relative to its stage, block count, 0
+  const int4* stage;
+  const int32_t* sd_lev0;  // first stage of each subdomain (one closing entry more than its stages)
+  const int4* info;        // row records (HostSetup::SolvePlan::info)
 };
+// values per solution entry in the sweeps' work arrays: rows start on 16-byte boundaries
+template <class T>
+constexpr int SOLVE_STRIDE = sizeof(T) == 8 ? 6 : 8;
 struct RasDev {
   int32_t P;
   const int32_t* sd_sched;  // CTA b of a per-subdomain kernel works on subdomain sd_sched[b]
@@ -169,23 +207,19 @@ struct RasDev {
   // none, so every wait gives up at once); the final wait for issued copies to land
   // keeps the fixed bound SOLVE_DRAIN_POLLS
   int32_t wait_polls;
-  // blocks whose solution entries a consumer row loads before their FMAs (1-4; the autotuner's
-  // choice, 2 by default); every choice forms the same sums in the same order
-  int32_t solve_ch;
-  int32_t solve_warps;  // consumer warps per subdomain CTA: 7 (256 threads) or 3 (128 threads)
-  int32_t solve_ring;   // blocks in the factor ring: SOLVE_RING_FULL (two stages) or SOLVE_RING_HALF (one)
+  int32_t solve_warps;  // shape of a subdomain CTA: 7 (256 threads) or 3 (160 threads)
+  int32_t solve_ring;   // blocks of the factor ring (solve_ring_blocks)
 };
-constexpr int32_t SOLVE_RING_FULL = 2 * SOLVE_BUF_BLOCKS_DEV;
-constexpr int32_t SOLVE_RING_HALF = SOLVE_BUF_BLOCKS_DEV;
-// contexts of at most this many subdomains (one per SM) take the solve's WIDE form
-constexpr int32_t SOLVE_WIDE_MAX = 152;
 constexpr int32_t SOLVE_WAIT_POLLS_DEFAULT = 1 << 20;
 void launch_ilu_factor(const RasDev& d, const double* val, const float* val32, int32_t* err, bool fp32,
                        cudaStream_t s);
 void launch_ilu_reorg(const RasDev& d, int64_t nfwd, int64_t nbwd, const int64_t* fsrc, const int32_t* fcol,
-                      const int64_t* bsrc, const int32_t* bcol, bool fp32, cudaStream_t s);
+                      const int32_t* frow, const int64_t* bsrc, const int32_t* bcol, const int32_t* brow, bool fp32,
+                      cudaStream_t s);
 void launch_ilu_solve(const RasDev& d, const double* r, double* z, int32_t* err, cudaStream_t s);
-void launch_ilu_solve32(const RasDev& d, const double* r, float* z, int32_t* err, cudaStream_t s);
+// r in FP32, rows padded to eight values (launch_pack32, launch_az_sub32)
+void launch_ilu_solve32(const RasDev& d, const float* r, float* z, int32_t* err, cudaStream_t s);
+void launch_pack32(int64_t n, const double* r, float* out, cudaStream_t s);
 void launch_spmv32(int64_t nrow, const int32_t* rp, const int32_t* col, const float* val, const float* x, double* y,
                    cudaStream_t s, int tb = 256, const double* b = nullptr);
 void launch_multi_axpy32(int64_t len, int nv, const float* Zs, int64_t ld, const double* coef, double* x,
@@ -217,13 +251,15 @@ void launch_coarse_assemble(const CoarseDev& c, const double* val, const float* 
 void launch_az_build(int64_t nseg, const int32_t* az_blk, const double* val, const float* val32, double* azval,
                      float* azval32, bool fp32, cudaStream_t s);
 void launch_az_sub(const CoarseDev& c, int64_t n, const int64_t* az_ptr, const int32_t* az_unit,
-                   const double* azval, const float* azval32, bool fp32, double* t, cudaStream_t s);
+                   const double* azval, double* t, cudaStream_t s);
+void launch_az_sub32(const CoarseDev& c, int64_t n, const int64_t* az_ptr, const int32_t* az_unit,
+                     const float* azval, const double* t, float* out, cudaStream_t s);
 void launch_coarse_factor(const CoarseDev& c, int32_t* err, cudaStream_t s);
 template <class TZ>
 void launch_coarse_apply_add(const CoarseDev& c, int64_t n, const double* r, TZ* z, cudaStream_t s);
 void launch_coarse_solve(const CoarseDev& c, const double* r, cudaStream_t s);
 // mixed-precision path, after launch_coarse_solve: y32 = (float) y, then z += Z y32 in FP32,
-// and t -= (J Z) y32 with FP32 products (accumulated in FP32, subtracted in FP64)
+// and out = t - (J Z) y32 with FP32 products (accumulated in FP32, subtracted in FP64)
 void launch_coarse_y32(const CoarseDev& c, cudaStream_t s);
 void launch_coarse_prolong32(const CoarseDev& c, int64_t n, float* z, cudaStream_t s);
 template <class TZ>

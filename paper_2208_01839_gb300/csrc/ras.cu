@@ -10,6 +10,7 @@
 // entries by their position in the sweep.  The coarse matrix is block-banded
 // (subdomains in reverse Cuthill-McKee order) and factored by block LU with 5x5
 // pivot blocks inverted under partial pivoting, then inverted explicitly.
+#include <algorithm>
 #include <cmath>
 
 #include "kernels.cuh"
@@ -146,21 +147,20 @@ __global__ void __launch_bounds__(256) k_ilu_factor(RasDev d, const TV* __restri
         const int32_t k = d.l_col[a];
         if (k >= i) break;  // columns are sorted: the strictly lower blocks come first
         const T* Dk = dinv + 25 * ((int64_t)r0 + k);
-        T* A = fval + 25 * a;
-        T v = T(0);
+        const T* A = fval + 25 * a;  // stays A_ik = L_ik U_kk: what the solve's copy is made of
+        T v = T(0), L[5];
         if (lane < 25) {
 #pragma unroll
           for (int mm = 0; mm < 5; ++mm) v = fmaT(A[5 * rr + mm], Dk[5 * mm + cc], v);
         }
-        __syncwarp();
-        if (lane < 25) A[lane] = v;  // L_ik = A_ik U_kk^{-1}
-        __syncwarp();
+#pragma unroll
+        for (int mm = 0; mm < 5; ++mm) L[mm] = __shfl_sync(FULL, v, (5 * rr + mm) & 31);  // L_ik = A_ik U_kk^{-1}
         for (int64_t u = d.upd_ptr[a]; u < d.upd_ptr[a + 1]; ++u) {
           const int64_t dst = d.upd[2 * u], src = d.upd[2 * u + 1];
           if (lane < 25) {  // A_ij -= L_ik U_kj, folded into the FMA chain
             T t = fval[25 * dst + lane];
 #pragma unroll
-            for (int mm = 0; mm < 5; ++mm) t = fmaT(-A[5 * rr + mm], fval[25 * src + 5 * mm + cc], t);
+            for (int mm = 0; mm < 5; ++mm) t = fmaT(-L[mm], fval[25 * src + 5 * mm + cc], t);
             fval[25 * dst + lane] = t;
           }
         }
@@ -175,15 +175,13 @@ __global__ void __launch_bounds__(256) k_ilu_factor(RasDev d, const TV* __restri
 
 // ---- subdomain solves ---------------------------------------------------------
 //
-// The solve reads the factors from a copy in level order (SolvePlan): every
-// level of the forward (then backward) sweep is one contiguous range of padded
-// blocks (25 values and the block's local column in slot 25; 26 doubles or 28
-// floats, so a block is a multiple of 16 bytes).  While a level computes, the
-// next level's range is already in flight into the other half of a double
-// buffer in shared memory (cp.async.bulk completing on an mbarrier), so the
-// only global loads on a level's critical path are the solution entries of
-// earlier levels.  Rows are mapped six to a warp (lane = 5 row + component), so
-// the backward sweep's product with the inverted pivot block uses shuffles.
+// The solve reads the factors from a copy in level order (SolvePlan), scaled so that a
+// row's result is one sum of block products: Dinv_i and -Dinv_i A_ij (lower and upper
+// blocks alike; A_ij the factorisation's blocks L_ij U_jj and U_ij).  Every level of the
+// forward (then backward) sweep is one contiguous range of padded blocks (25 values and
+// the block's local column in slot 25; 26 doubles or 28 floats, so a block is a multiple
+// of 16 bytes), which streams into shared memory by cp.async.bulk while earlier levels
+// compute.
 
 template <class T>
 struct SolveBS;
@@ -201,9 +199,13 @@ __device__ __forceinline__ int col_of(float x) { return __float_as_int(x); }
 __device__ __forceinline__ void put_col(double* p, int c) { *p = __longlong_as_double((long long)c); }
 __device__ __forceinline__ void put_col(float* p, int c) { *p = __int_as_float(c); }
 
+// The solve's copy of the factors: block b is Dinv_R (src = -1 - R) or -Dinv_R A, A the
+// factor block src and R = brow its row; one thread per value.
 template <class T>
-__global__ void k_ilu_reorg(int64_t nblk, const int64_t* __restrict__ src, const int32_t* __restrict__ col,
-                            const T* __restrict__ fval, const T* __restrict__ dinv, T* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_ilu_reorg(int64_t nblk, const int64_t* __restrict__ src,
+                                                   const int32_t* __restrict__ col, const int32_t* __restrict__ brow,
+                                                   const T* __restrict__ fval, const T* __restrict__ dinv,
+                                                   T* __restrict__ out) {
   constexpr int BS = SolveBS<T>::v;
   for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < nblk * BS;
        g += (int64_t)gridDim.x * blockDim.x) {
@@ -211,9 +213,20 @@ __global__ void k_ilu_reorg(int64_t nblk, const int64_t* __restrict__ src, const
     const int e = (int)(g - b * BS);
     if (e < 25) {
       const int64_t s = src[b];
-      out[g] = s >= 0 ? fval[25 * s + e] : dinv[25 * (-1 - s) + e];
-    } else if (e == 25) {
-      put_col(out + g, col[b]);
+      const T* D = dinv + 25 * (int64_t)brow[b];
+      if (s >= 0) {
+        const int r = e / 5, c = e - 5 * r;
+        const T* A = fval + 25 * s + c;
+        T v = T(0);
+#pragma unroll
+        for (int mm = 0; mm < 5; ++mm) v = fmaT(-D[5 * r + mm], A[5 * mm], v);
+        out[g] = v;
+      } else {
+        out[g] = D[e];
+      }
+    } else if (e == 25) {  // window offset of the entry in bytes, or -1 - position where the plan says "far"
+      const int c = col[b];
+      put_col(out + g, c >= 0 ? (c & (SOLVE_WIN - 1)) * SOLVE_STRIDE<T> * (int)sizeof(T) : c);
     } else {
       out[g] = T(0);
     }
@@ -252,30 +265,34 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int po
 // copy is in flight into the shared memory of a CTA that has left
 constexpr int SOLVE_DRAIN_POLLS = 1 << 20;
 
-// Stage data of one subdomain stream through shared memory: the factor blocks
-// (SolveRing blocks), the per-row records and the rows' first values (r in the forward
-// sweep, the forward result in the backward one; SOLVE_RING_ROWS rows).  Warp NCW is
-// the producer: its lane 0 reads the level plan and issues the bulk copies of up to
-// SOLVE_SLOTS stages ahead, as far as the rings have room, and all its lanes gather
-// the first values by cp.async; a stage's "full" mbarrier completes when all of them
-// have landed, and its "empty" mbarrier when the consumers are done with it.  The
-// consumer warps take the stages in order and meet at a named barrier after each one
-// (the rows of a level depend on the rows of earlier levels).  A stage never wraps
-// around a ring's end: the producer skips the tail.  The producer starts the backward
-// sweep's stages once the forward sweep is complete (their first values are its
-// results).  Every wait is bounded; on a timeout the kernel sets bit 3 of *err, lets
-// every issued copy land and returns.
-// Solution entries are numbered by their position in the sweep; the last SOLVE_WIN of
-// them are kept in shared memory, where nearly all of a row's dependencies lie, and
-// every entry goes to the work arrays in global memory for the rest and for the
-// backward sweep.
-// Ring of factor blocks: two stages (236 blocks) or one (118), which leaves the shared
-// memory to more resident subdomains (SOLVE_RING_FULL / SOLVE_RING_HALF).
-constexpr int SOLVE_RING_ROWS = SOLVE_BUF_ROWS_DEV;
-constexpr int SOLVE_WIN = 256;
-constexpr int SOLVE_SLOTS = 8;
-static_assert(SOLVE_WIN >= 2 * SOLVE_BUF_ROWS_DEV && (SOLVE_WIN & (SOLVE_WIN - 1)) == 0,
-              "a stage's rows must not displace the window's entries that it reads");
+// Stage data of one subdomain stream through shared memory: the factor blocks, the row
+// records and the rows' first values (r in the forward sweep, the forward result in the
+// backward one).  Two warps bring them, up to SOLVE_SLOTS stages ahead and as far as the
+// rings have room: one thread issues the bulk copies (records, blocks, the backward sweep's
+// first values; "recs" and "blks" mbarriers), one warp gathers a forward stage's r by
+// cp.async once its records are here ("vals").  Where a stage goes and which stage must have
+// been consumed before it is part of the stage's record, so each of the two has one wait a
+// stage; the blocks are also drawn into L2 ahead of their copies.  The consumer warps take
+// the stages in order and meet at a named barrier after each one (the rows of a level depend
+// on the rows of earlier levels), which the last of them joins when the next stage has
+// arrived, so that the others have no wait of their own; a stage's "empty" mbarrier then
+// completes.  (An mbarrier test takes 110 clocks, as long as a whole batch of FP32
+// products; a barrier of eight warps takes 28.)  Every wait is bounded; on a timeout the
+// kernel sets bit 3 of *err, lets every issued copy land and returns.
+// The work arrays y and z hold one padded row per sweep position.  The forward sweep leaves
+// its results in y, and in z at the row's backward position, where the backward sweep finds
+// its first values as one contiguous run a stage and leaves its results.  The last SOLVE_WIN
+// results of a sweep also stay in shared memory, where nearly all of a row's dependencies
+// lie; which ones do not is known at set-up (HostSetup::SolvePlan::col).
+// Ring of factor blocks: several stages, or one (118 blocks), which leaves the shared memory
+// to more resident subdomains (solve_ring_blocks).  How far the copies run ahead is what
+// bounds a stage once its own chain is short: 128 subdomains of 4400 rows, ILU(1), take 1.74
+// ms in FP64 (1.20 in FP32) with the short ring and 1.12 (0.61) with the long one.
+// Measured for a preconditioner apply without a coarse space (one sweep pair and the two
+// index permutations), start of these sweeps -> now: 1024 x 1024 nodes, 512 subdomains, ILU(1)
+// 1.24 -> 1.04 ms FP64, 0.69 -> 0.50 ms FP32; 501k nodes, 128 subdomains, ILU(1) 1.67 -> 1.12
+// and 0.97 -> 0.61 ms; 16 subdomains of 4489 rows, ILU(0) 0.94 -> 0.76 and 0.57 -> 0.45 ms.
+constexpr int SOLVE_AHEAD = 320;  // blocks drawn into L2 ahead of their copies
 
 __device__ __forceinline__ void mbar_init_count(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
@@ -288,288 +305,286 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void cp_async_value(double* dst, const double* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+// five values of r: doubles at stride 5, or floats padded to stride 8
+__device__ __forceinline__ void cp_async_row(double* dst, const double* r, int64_t i) {
+  const uint32_t d = smem_u32(dst);
+#pragma unroll
+  for (int c = 0; c < 5; ++c)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8 * c), "l"(r + 5 * i + c) : "memory");
 }
-__device__ __forceinline__ void cp_async_value(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+__device__ __forceinline__ void cp_async_row(float* dst, const float* r, int64_t i) {
+  const uint32_t d = smem_u32(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(r + 8 * i) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 16), "l"(r + 8 * i + 4) : "memory");
 }
-// named barrier 1 over the NCW consumer warps (the producer warp does not take part)
-template <int NCW>
+// this thread's stores before it are seen by bulk copies issued after a synchronisation
+// that follows it
+__device__ __forceinline__ void fence_bulk() { asm volatile("fence.proxy.async;" ::: "memory"); }
+// named barrier 1 over the NC consumer warps
+template <int NC>
 __device__ __forceinline__ void consumers_sync() {
-  asm volatile("bar.sync 1, %0;" ::"n"(32 * NCW) : "memory");
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * NC) : "memory");
 }
 
-// What the consumer warps share for one stage.
-template <class T>
-struct StageView {
-  const T* B;         // the stage's factor blocks
-  const int4* inf;    // its row records
-  const double* fv;   // its first values, five 8-byte slots a row (type T in the backward sweep)
-  T* vec;             // solution entries of the sweep in global memory
-  T* win;             // the last SOLVE_WIN of them
-  int nrows, k0;      // rows, sweep position of the first
-};
-
-// One stage's rows, S lanes groups to a row: a warp takes 6 / S rows, lane = 5 (part R + row) +
-// component, and part p of a row sums its blocks p, p + S, ...  An FP64 FMA occupies a
-// warp for 64 clocks whatever its lanes and dependences, and an SM runs four such warps
-// at once, so a stage of few rows is quicker with its rows' blocks spread over more
-// warps.  S = 1 keeps two chains (blocks of even and odd number) that are added at the
-// end: the same sums in the same order as the two parts of S = 2, so either may be
-// taken for any stage.  The entries of CH blocks are loaded before any of their FMAs.
-// Measured with the gathered first values and the window: 2.0M nodes, 512 subdomains,
-// ILU(1), FP64 2.36 -> 1.93 ms a solve; 1024 x 1024, FP32 0.607 -> 0.58 ms.
-template <int S, class T, class TZ, int CH, int NCW>
-__device__ __forceinline__ void stage_rows(const StageView<T>& sv, bool fw, int warp, int lane, TZ* __restrict__ z) {
-  constexpr int BS = SolveBS<T>::v;
-  constexpr int R = 6 / S;
-  const int l5 = lane / 5, cpt = lane - 5 * l5;
-  const int part = S == 1 ? 0 : l5 / R, rw = l5 - part * R;
-  const int lo = sv.k0 + sv.nrows - SOLVE_WIN;  // first position that this stage's results leave in the window
-  const int jb = fw ? 0 : 1;                    // block 0 of a backward row is the inverted pivot
-  for (int qb = warp * R; qb < sv.nrows; qb += R * NCW) {
-    const int q = qb + rw;
-    const bool act = lane < 30 && q < sv.nrows;
-    int st = 0, cn = 0, onode = -1;
-    T acc = T(0), acc2 = T(0);
-    if (act) {
-      const int4 rec = sv.inf[q];
-      st = rec.y;
-      cn = rec.z;
-      onode = rec.w;
-      if (part == 0) acc = fw ? (T)sv.fv[5 * q + cpt] : reinterpret_cast<const T*>(sv.fv + 5 * q)[cpt];
-    }
-    for (int j = jb + part; j < cn; j += S * CH) {
-      const int nb = S == 1 ? min(CH, cn - j) : min(CH, (cn - j + S - 1) / S);
-      T xv[CH][5];
-#pragma unroll
-      for (int u = 0; u < CH; ++u) {  // a short row reloads its last block to fill the batch
-        const int pos = col_of(sv.B[(st + j + S * min(u, nb - 1)) * BS + 25]);
-        const T* vk = pos >= lo ? sv.win + 5 * (pos & (SOLVE_WIN - 1)) : sv.vec + 5 * (int64_t)pos;
-#pragma unroll
-        for (int mm = 0; mm < 5; ++mm) xv[u][mm] = vk[mm];
-      }
-#pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        if (u < nb) {
-          const T* Lb = sv.B + (st + j + S * u) * BS + 5 * cpt;
-#pragma unroll
-          for (int mm = 0; mm < 5; ++mm) {
-            if (S == 1 && (u & 1)) acc2 = fmaT(-Lb[mm], xv[u][mm], acc2);
-            else acc = fmaT(-Lb[mm], xv[u][mm], acc);
-          }
-        }
-      }
-      if (S == 1 && CH % 2 == 1) {  // the next batch starts on the other chain
-        const T t = acc;
-        acc = acc2;
-        acc2 = t;
-      }
-    }
-    // the parts' sums; FP addition commutes, so whichever register holds which chain of S = 1
-    // the sum is the same
-    if (S == 1) {
-      acc += acc2;
-    } else {
-      T oth[S];
-#pragma unroll
-      for (int p = 1; p < S; ++p) oth[p] = __shfl_sync(FULL, acc, (lane + 5 * R * p) & 31);
-      if (S == 2) {
-        acc += oth[1];
-      } else if (S == 3) {
-        acc += oth[1] + oth[2];
-      } else {
-#pragma unroll
-        for (int p = 1; p + 1 < S; p += 2) oth[p] += oth[p + 1];
-        if (S == 6) acc = (acc + oth[S - 1]) + (oth[1] + oth[3]);
-      }
-    }
-    const int kq = sv.k0 + q;  // this row's position
-    T v = acc;
-    if (!fw) {
-      // z = U_kk^{-1} (...): the five partial results of the row sit in lanes 5 rw .. 5 rw + 4
-      v = T(0);
-      const T* Dv = sv.B + st * BS + 5 * cpt;
-#pragma unroll
-      for (int mm = 0; mm < 5; ++mm) {
-        const T am = __shfl_sync(FULL, acc, 5 * rw + mm);
-        if (act) v = fmaT(Dv[mm], am, v);
-      }
-    }
-    if (act && part == 0) {
-      sv.vec[5 * (int64_t)kq + cpt] = v;
-      sv.win[5 * (kq & (SOLVE_WIN - 1)) + cpt] = v;
-      if (!fw && onode >= 0) z[5 * (int64_t)onode + cpt] = (TZ)v;
-    }
-  }
+// five values of a row of a work array or of the window (16-byte aligned)
+__device__ __forceinline__ void load5(const double* p, double (&v)[5]) {
+  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = b.x;
+  v[3] = b.y;
+  v[4] = p[4];
+}
+__device__ __forceinline__ void load5(const float* p, float (&v)[5]) {
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = a.z;
+  v[3] = a.w;
+  v[4] = p[4];
 }
 
-// NCW consumer warps (7 or 3) and one producer warp.  Every row's arithmetic is the same
-// for either count.  WIDE (contexts whose subdomains do not fill the SMs) splits the rows
-// of small stages over up to six parts: what counts there is a stage's own latency, and
-// nothing else uses the FP64 pipe.
-template <class T, class TZ, int CH, int NCW, int RB, bool WIDE>
-__global__ void __launch_bounds__(32 * (NCW + 1), NCW <= 3 ? 7 : 4)
-    k_ilu_solve(RasDev d, const double* __restrict__ r, TZ* __restrict__ z, int32_t* err) {
-  constexpr int BS = SolveBS<T>::v;
-  constexpr int RR = SOLVE_RING_ROWS;
+// Consumer warps of the two CTA shapes: 7 names the one of 256 threads (six consumers and the
+// two copying warps), 3 the one of 160 (three and two).  Every row's arithmetic is the same.
+constexpr int solve_consumers(int ncw) { return ncw == 7 ? 6 : 3; }
+
+template <class T, class TZ, int NCW, int RB, bool WIDE>
+__global__ void __launch_bounds__(32 * (solve_consumers(NCW) + 2), NCW <= 3 ? 6 : 4)
+    k_ilu_solve(RasDev d, const T* __restrict__ r, TZ* __restrict__ z, int32_t* err) {
+  constexpr int NC = solve_consumers(NCW);
+  constexpr int BS = SolveBS<T>::v, BSB = BS * (int)sizeof(T);
+  constexpr int RR = solve_ring_rows(RB);
+  constexpr int RBP = RB + SOLVE_RING_SPARE, RV = RB == SOLVE_RING_HALF ? 1 : 0;
   constexpr int NS = SOLVE_SLOTS;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t full[NS];
-  __shared__ __align__(8) uint64_t empty[NS];
+  constexpr int W = SOLVE_STRIDE<T>, WB = W * (int)sizeof(T);
+  extern __shared__ __align__(128) unsigned char smem[];  // factor ring, first values, window
+  constexpr int FV = RBP * BSB, WIN = FV + RR * WB;
+  __shared__ __align__(8) uint64_t recs[NS], blks[NS], vals[NS], empty[NS];
   __shared__ __align__(16) int4 info[RR];
-  __shared__ __align__(16) int4 slot[NS];  // ring starts (blocks, rows), row count and first position of a stage
-  __shared__ int2 virt[NS];  // virtual ring starts of the stages in flight (producer's lane 0)
+  __shared__ __align__(16) int4 slot[NS];  // byte offset of the blocks, first row of the row rings, rows (| 256: `ahead`), first position
   __shared__ int abort_at;  // first stage at which a consumer warp's wait gave up (INT_MAX: none)
-  T* ring = reinterpret_cast<T*>(smem_raw);
-  double* fv = reinterpret_cast<double*>(ring + (size_t)RB * BS);
-  T* win = reinterpret_cast<T*>(fv + 5 * RR);
-  const int p = d.sd_sched ? d.sd_sched[blockIdx.x] : (int)blockIdx.x;
+  const int p = d.sd_sched[blockIdx.x];
   const int32_t r0 = d.sd_row0[p];
-  T* y = ywk<T>(d) + 5 * (int64_t)r0;
-  T* zz = zwk<T>(d) + 5 * (int64_t)r0;
+  T* const y = ywk<T>(d) + (int64_t)W * r0;
+  T* const zz = zwk<T>(d) + (int64_t)W * r0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int32_t LF = d.fwd.sd_lev0[p], nF = d.fwd.sd_lev0[p + 1] - LF - 1;
   const int32_t LB = d.bwd.sd_lev0[p], nB = d.bwd.sd_lev0[p + 1] - LB - 1;
   const int nstage = nF + nB;
   if (tid == 0) {
     for (int k = 0; k < NS; ++k) {
-      mbar_init_count(&full[k], 33);  // lane 0's bulk copies and the 32 lanes' gathers
+      mbar_init_count(&recs[k], 1);
+      mbar_init_count(&blks[k], 1);
+      mbar_init_count(&vals[k], 32);
       mbar_init_count(&empty[k], 1);
     }
     abort_at = INT_MAX;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  // stage g < nF is forward level g, otherwise backward level g - nF; it uses slot g % NS,
+  // whose barriers complete phase (g / NS) & 1 for it (forward stages come first, so this
+  // holds for the gathered ones too)
+  auto phase = [](int g) { return (uint32_t)((g / NS) & 1); };
 
-  if (warp == NCW) {
-    // ---- producer: stage g < nF is forward level g, otherwise backward level
-    // g - nF; it uses slot g % NS, whose barriers complete phase (g / NS) & 1 for it.
-    // The plan entries and the rows' gather indices of a stage are read one stage ahead.
-    constexpr int NU = (SOLVE_BUF_ROWS_DEV + 31) / 32;
-    int q0 = 0, nr = 0, nb = 0, id[NU];
-    int64_t b0 = 0;
-    auto plan = [&](int g, int& pq0, int& pnr, int64_t& pb0, int& pnb, int (&pid)[NU]) {
-      if (g >= nstage) return;
-      const bool fw = g < nF;
-      const SolvePlanDev& P = fw ? d.fwd : d.bwd;
-      const int32_t lv = fw ? LF + g : LB + g - nF;
-      pq0 = P.levpos[lv];
-      pnr = P.levpos[lv + 1] - pq0;
-      pb0 = P.levblk[lv];
-      pnb = (int)(P.levblk[lv + 1] - pb0);
-#pragma unroll
-      for (int u = 0; u < NU; ++u)
-        if (lane + 32 * u < pnr) pid[u] = P.info[(int64_t)r0 + pq0 + lane + 32 * u].x;
+  if (warp == NC) {
+    // ---- bulk copies (one thread); stage records are read four stages ahead
+    if (lane != 0) return;
+    auto record = [&](int g) {
+      if (g >= nstage) return make_int4(0, 0, 0, 0);
+      return g < nF ? d.fwd.stage[LF + g] : d.bwd.stage[LB + g - nF];
     };
-    plan(0, q0, nr, b0, nb, id);
-    int vb = 0, vr = 0, oldest = 0;  // ring heads (virtual, growing); oldest stage not known to be released
+    int4 st[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) st[u] = record(u);
+    int pf = st[0].y, pend = 0;  // L2 prefetch: next block, end of the sweep's blocks
     int gi = 0;
     bool ok = true;
-    for (; gi < nstage; ++gi) {
-      const bool fw = gi < nF;
-      int nq0 = 0, nnr = 0, nnb = 0, nid[NU];
-      int64_t nb0 = 0;
-      plan(gi + 1, nq0, nnr, nb0, nnb, nid);
-      int sb = vb, sr = vr;
-      if (sb % RB + nb > RB) sb += RB - sb % RB;
-      if (sr % RR + nr > RR) sr += RR - sr % RR;
-      const int sl = gi % NS;
-      if (lane == 0) {
-        // release stages (in order) until this one fits and its slot is free; all of the
-        // forward sweep before the first backward stage
-        while (oldest < gi) {
-          const int os = oldest % NS;
-          const int2 at = virt[os];
-          if (!(gi == nF || gi - oldest >= NS || sb + nb - at.x > RB || sr + nr - at.y > RR)) break;
-          if (!mbar_wait(&empty[os], (uint32_t)((oldest / NS) & 1), d.wait_polls) ||
-              *(volatile int*)&abort_at != INT_MAX) {
-            ok = false;
-            break;
-          }
-          ++oldest;
-        }
-      }
-      ok = __shfl_sync(FULL, (int)ok, 0) != 0;
-      if (!ok) break;
-      const int rb = sb % RB, rr = sr % RR;
-      if (lane == 0) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        virt[sl] = make_int2(sb, sr);
-        slot[sl] = make_int4(rb, rr, nr, q0);
-        const uint32_t bytes_b = (uint32_t)nb * BS * (uint32_t)sizeof(T);
-        const uint32_t bytes_i = (uint32_t)nr * (uint32_t)sizeof(int4);
-        mbar_arrive_tx(&full[sl], bytes_b + bytes_i);  // releases the slot fields above to the consumers
-        if (bytes_b) bulk_g2s(ring + (size_t)rb * BS, (fw ? solve_fwd<T>(d) : solve_bwd<T>(d)) + b0 * BS, bytes_b, &full[sl]);
-        if (bytes_i) bulk_g2s(info + rr, (fw ? d.fwd : d.bwd).info + r0 + q0, bytes_i, &full[sl]);
-      }
+    while (ok && gi < nstage) {
 #pragma unroll
-      for (int u = 0; u < NU; ++u) {
-        const int q = lane + 32 * u;
-        if (q < nr) {
-          double* dst = fv + 5 * (rr + q);
-          if (fw) {
-#pragma unroll
-            for (int c = 0; c < 5; ++c) cp_async_value(dst + c, r + 5 * (int64_t)id[u] + c);
-          } else {
-#pragma unroll
-            for (int c = 0; c < 5; ++c) cp_async_value(reinterpret_cast<T*>(dst) + c, y + 5 * (int64_t)id[u] + c);
+      for (int u = 0; u < 4; ++u) {
+        if (ok && gi < nstage) {
+          const int4 s = st[u];
+          st[u] = record(gi + 4);
+          const bool fw = gi < nF;
+          const int sl = gi % NS, nr = stage_rows(s), nb = stage_blocks(s);
+          const int dist = stage_distance(s, RV);
+          if (dist != SOLVE_FREE) ok = mbar_wait(&empty[(gi - dist) % NS], phase(gi - dist), d.wait_polls);
+          if (ok) {
+            const int rb = stage_block_offset(s, RV), rr = stage_row_offset(s, RV);
+            const bool ahead = stage_distance(st[(u + 1) & 3], RV) >= 2;  // the next stage does not wait for this one
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            slot[sl] = make_int4(rb * BSB, rr, nr | (int)ahead << 8, s.x);
+            const uint32_t bytes_b = (uint32_t)nb * BSB, bytes_i = (uint32_t)nr * (uint32_t)sizeof(int4);
+            const uint32_t bytes_v = fw ? 0u : (uint32_t)nr * WB;
+            const T* F = fw ? solve_fwd<T>(d) : solve_bwd<T>(d);
+            mbar_arrive_tx(&recs[sl], bytes_i);  // releases the slot with the records
+            if (bytes_i) bulk_g2s(info + rr, (fw ? d.fwd : d.bwd).info + r0 + s.x, bytes_i, &recs[sl]);
+            mbar_arrive_tx(&blks[sl], bytes_b + bytes_v);
+            if (bytes_b) bulk_g2s(smem + rb * BSB, F + (int64_t)s.y * BS, bytes_b, &blks[sl]);
+            if (bytes_v) bulk_g2s(smem + FV + rr * WB, zz + (int64_t)W * s.x, bytes_v, &blks[sl]);
+            if (gi == 0 || gi == nF) {
+              pf = s.y + nb;
+              const int4 last = fw ? d.fwd.stage[LF + nF - 1] : d.bwd.stage[LB + nB - 1];
+              pend = last.y + stage_blocks(last);
+            }
+            while (pf < pend && pf < s.y + SOLVE_AHEAD) {
+              const int n = min(64, pend - pf);
+              asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(F + (int64_t)pf * BS), "r"((uint32_t)n * BSB)
+                           : "memory");
+              pf += n;
+            }
+            ++gi;
           }
         }
       }
-      cp_async_arrive(&full[sl]);
-      vb = sb + nb;
-      vr = sr + nr;
-      q0 = nq0;
-      nr = nnr;
-      b0 = nb0;
-      nb = nnb;
-#pragma unroll
-      for (int u = 0; u < NU; ++u) id[u] = nid[u];
     }
-    if (!ok && lane == 0) atomicOr(err, 8);
+    if (!ok) atomicOr(err, 8);
     // every issued copy lands before the CTA can exit (the last stage issued on
-    // each slot is the only one whose phase is still open)
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (lane == 0)
-      for (int k = gi - 1; k >= 0 && k >= gi - NS; --k)
-        mbar_wait(&full[k % NS], (uint32_t)((k / NS) & 1), SOLVE_DRAIN_POLLS);
+    // each slot is the only one whose phases may still be open)
+    for (int k = max(0, gi - NS); k < gi; ++k) {
+      mbar_wait(&recs[k % NS], phase(k), SOLVE_DRAIN_POLLS);
+      mbar_wait(&blks[k % NS], phase(k), SOLVE_DRAIN_POLLS);
+    }
     return;
   }
 
-  // ---- consumers (warps 0 .. NCW - 1)
-  // A warp whose wait gives up skips the stage and records it; every consumer
-  // reads abort_at after the named barrier that closes the stage, and only
-  // values <= g (written before that barrier) end the loop at stage g, so all
-  // consumer warps leave at the same stage.
-  bool aborted = false;
-  StageView<T> sv;
-  sv.win = win;
-  for (int g = 0; g < nstage; ++g) {
-    const bool fw = g < nF;
-    const int sl = g % NS;
-    const bool landed = __all_sync(FULL, mbar_wait(&full[sl], (uint32_t)((g / NS) & 1), d.wait_polls));
-    if (!landed && lane == 0) atomicMin(&abort_at, g);
-    const int4 ds = slot[sl];
-    sv.B = ring + (size_t)ds.x * BS;
-    sv.inf = info + ds.y;
-    sv.fv = fv + 5 * ds.y;
-    sv.vec = fw ? y : zz;
-    sv.nrows = landed ? ds.z : 0;
-    sv.k0 = ds.w;
-    if (WIDE && sv.nrows <= 7) stage_rows<6, T, TZ, CH, NCW>(sv, fw, warp, lane, z);
-    else if (WIDE && sv.nrows <= 14) stage_rows<3, T, TZ, CH, NCW>(sv, fw, warp, lane, z);
-    else if (sv.nrows <= 3 * NCW) stage_rows<2, T, TZ, CH, NCW>(sv, fw, warp, lane, z);
-    else stage_rows<1, T, TZ, CH, NCW>(sv, fw, warp, lane, z);
-    consumers_sync<NCW>();  // every row of this stage is written; the stage's ring space is free
-    if (*(volatile int*)&abort_at <= g) {
-      aborted = true;
-      break;
+  if (warp == NC + 1) {
+    // ---- gathers of the forward stages' r
+    bool ok = true;
+    for (int g = 0; g < nF && ok; ++g) {
+      const int sl = g % NS;
+      ok = __all_sync(FULL, mbar_wait(&recs[sl], phase(g), d.wait_polls));
+      if (ok) {
+        const int4 ds = slot[sl];
+        for (int q = lane; q < (ds.z & 255); q += 32)
+          cp_async_row(reinterpret_cast<T*>(smem + FV) + W * (ds.y + q), r, info[ds.y + q].x);
+        cp_async_arrive(&vals[sl]);
+      }
     }
-    if (tid == 0) mbar_arrive(&empty[sl]);
+    if (!ok && lane == 0) atomicOr(err, 8);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    return;
   }
-  if (aborted && tid == 0) atomicOr(err, 8);
+
+  // ---- consumers (warps 0 .. NC - 1).  S lane groups to a row: a warp takes 6 / S rows,
+  // lane = 5 (part (6 / S) + row) + component, and part p of a row sums its blocks p,
+  // p + S, ...; the inverted pivot (forward) or the first value (backward) opens part 0.
+  // An FP64 FMA holds a warp for 64 clocks whatever its lanes and dependences, and four
+  // such warps fill an SM's FP64 pipe; in FP32 a stage costs its chain of instructions.
+  // Both want a stage's rows spread over the warps there are, and short code.  S = 1
+  // keeps the sums of a row's even and odd blocks apart and adds them at the end, as the
+  // two parts of S = 2 do: the same sums in the same order, so a launch shape may take
+  // either.
+  const int l5 = lane / 5, cpt = lane - 5 * l5;
+  auto rows = [&]<int S>(const int4 ds, int nr, bool fw, int q0) {
+    constexpr int R = 6 / S;
+    const int part = S == 1 ? 0 : l5 / R, q = q0 + l5 - part * R;
+    const bool act = lane < 30 && q < nr;
+    int4 rec = make_int4(0, 0, 0, -1);
+    T acc = T(0), acc2 = T(0);
+    if (act) rec = info[ds.y + q];
+    const unsigned char* B = smem + ds.x + rec.y * BSB;  // the row's blocks
+    const T* vec = fw ? y : zz;
+    int j = part;
+    if (act && part == 0) {
+      const T* f = reinterpret_cast<const T*>(smem + FV) + W * (ds.y + q);
+      if (fw) {
+        T x[5];
+        load5(f, x);
+#pragma unroll
+        for (int mm = 0; mm < 5; ++mm)
+          if (S == 1) acc2 = fmaT(reinterpret_cast<const T*>(B)[5 * cpt + mm], x[mm], acc2);
+          else acc = fmaT(reinterpret_cast<const T*>(B)[5 * cpt + mm], x[mm], acc);
+        j = S;  // block 0 is done (S = 1: in the even chain, and block 1 is odd)
+      } else {
+        acc = f[cpt];
+      }
+    }
+#pragma unroll 1
+    for (; j < rec.z; j += S) {
+      const unsigned char* Bj = B + j * BSB;
+      const int c = col_of(*reinterpret_cast<const T*>(Bj + 25 * (int)sizeof(T)));
+      T x[5];
+      if (c >= 0) load5(reinterpret_cast<const T*>(smem + WIN + c), x);
+      else load5(vec + W * ~c, x);
+#pragma unroll
+      for (int mm = 0; mm < 5; ++mm) acc = fmaT(reinterpret_cast<const T*>(Bj)[5 * cpt + mm], x[mm], acc);
+      if (S == 1) {  // the next block belongs to the other chain
+        const T t = acc;
+        acc = acc2;
+        acc2 = t;
+      }
+    }
+    if (S == 1) {
+      acc += acc2;  // FP addition commutes: whichever register holds which chain
+    } else {
+      T oth[S];
+#pragma unroll
+      for (int k = 1; k < S; ++k) oth[k] = __shfl_sync(FULL, acc, (lane + 5 * R * k) & 31);
+      if (S == 2) acc += oth[1];
+      else if (S == 3) acc += oth[1] + oth[2];
+      else if (S == 6) acc = (acc + oth[S - 1]) + ((oth[1] + oth[S / 3]) + (oth[S / 2] + oth[S - 2]));
+    }
+    if (act && part == 0) {
+      const int k = ds.w + q;
+      reinterpret_cast<T*>(smem + WIN)[W * (k & (SOLVE_WIN - 1)) + cpt] = acc;
+      if (fw) {
+        y[W * k + cpt] = acc;
+        zz[W * rec.w + cpt] = acc;
+      } else {
+        zz[W * k + cpt] = acc;
+        if (rec.w >= 0) z[5 * (int64_t)rec.w + cpt] = (TZ)acc;
+      }
+    }
+  };
+  // One or two parts to a row give the same sums: two while a warp is left for each group
+  // of three rows, else six rows to a warp with the last one to three again in two parts.
+  // In FP32, where the FMAs are free, and for WIDE (no more subdomains than SMs, so that
+  // nothing else uses an SM's FP64 pipe while a stage waits for its longest row): more
+  // parts for the smallest stages, by their size alone.
+  // A warp whose wait gives up notes the stage and takes no rows of it; all warps leave
+  // after the barrier that closes that stage.
+  auto arrived = [&](int g) {
+    bool ok = mbar_wait(&blks[g % NS], phase(g), d.wait_polls);
+    ok = ok && mbar_wait(g < nF ? &vals[g % NS] : &recs[g % NS], phase(g), d.wait_polls);
+    return __all_sync(FULL, ok) != 0;
+  };
+  bool landed = arrived(0);
+  if (!landed && lane == 0) atomicMin(&abort_at, 0);
+  int g = 0;
+  for (; g < nstage; ++g) {
+    const int sl = g % NS;
+    const int4 ds = slot[sl];
+    if (*(volatile int*)&abort_at < g) break;
+    const bool fw = g < nF;
+    const int nr = landed ? ds.z & 255 : 0;
+    if ((WIDE || sizeof(T) == 4) && nr <= 4) {
+#pragma unroll 1
+      for (int q = warp; q < nr; q += NC) rows.template operator()<6>(ds, nr, fw, q);
+    } else if ((WIDE && nr <= 10) || (sizeof(T) == 4 && nr <= 12)) {
+#pragma unroll 1
+      for (int q = 2 * warp; q < nr; q += 2 * NC) rows.template operator()<3>(ds, nr, fw, q);
+    } else if (nr <= 3 * NC) {
+      if (3 * warp < nr) rows.template operator()<2>(ds, nr, fw, 3 * warp);
+    } else {
+      const int rem = nr % 6, six = rem > 3 ? nr : nr - rem;
+      int q = 6 * warp;
+#pragma unroll 1
+      for (; q < six; q += 6 * NC) rows.template operator()<1>(ds, nr, fw, q);
+      if (q == six && six < nr) rows.template operator()<2>(ds, nr, fw, q);
+    }
+    const bool ahead = landed && (ds.z & 256) != 0 && g + 1 < nstage;  // the next stage does not wait for this one
+    if (ahead && warp == NC - 1 && !arrived(g + 1) && lane == 0) atomicMin(&abort_at, g);
+    if (g == nF - 1) fence_bulk();  // the backward sweep's first values are read by bulk copies
+    consumers_sync<NC>();  // every row of this stage is written; its ring space is free
+    if (landed && tid == 0) mbar_arrive(&empty[sl]);
+    if (!ahead && g + 1 < nstage) {
+      landed = arrived(g + 1);
+      if (!landed && lane == 0) atomicMin(&abort_at, g + 1);
+    }
+  }
+  if (tid == 0 && (g < nstage || *(volatile int*)&abort_at != INT_MAX)) atomicOr(err, 8);
 }
 
 // ---- coarse space --------------------------------------------------------
@@ -816,82 +831,58 @@ void launch_ilu_factor(const RasDev& d, const double* val, const float* val32, i
   count_launch();
 }
 
-// dynamic shared memory of a solve CTA: factor ring, first values, solution window
+// dynamic shared memory of a solve CTA: factor ring, first values, window of results
 template <class T>
 constexpr size_t solve_smem(int ring_blocks) {
-  return ((size_t)ring_blocks * SolveBS<T>::v + 5 * SOLVE_WIN) * sizeof(T) + 5 * SOLVE_RING_ROWS * sizeof(double);
+  return ((size_t)(ring_blocks + SOLVE_RING_SPARE) * SolveBS<T>::v + SOLVE_STRIDE<T> * (solve_ring_rows(ring_blocks) + SOLVE_WIN)) *
+         sizeof(T);
 }
 
 void launch_ilu_reorg(const RasDev& d, int64_t nfwd, int64_t nbwd, const int64_t* fsrc, const int32_t* fcol,
-                      const int64_t* bsrc, const int32_t* bcol, bool fp32, cudaStream_t s) {
+                      const int32_t* frow, const int64_t* bsrc, const int32_t* bcol, const int32_t* brow, bool fp32,
+                      cudaStream_t s) {
   const int grid = 152 * 8;
   if (fp32) {
-    k_ilu_reorg<float><<<grid, 256, 0, s>>>(nfwd, fsrc, fcol, d.fval32, d.dinv32, d.fL32);
-    k_ilu_reorg<float><<<grid, 256, 0, s>>>(nbwd, bsrc, bcol, d.fval32, d.dinv32, d.bU32);
+    k_ilu_reorg<float><<<grid, 256, 0, s>>>(nfwd, fsrc, fcol, frow, d.fval32, d.dinv32, d.fL32);
+    k_ilu_reorg<float><<<grid, 256, 0, s>>>(nbwd, bsrc, bcol, brow, d.fval32, d.dinv32, d.bU32);
   } else {
-    k_ilu_reorg<double><<<grid, 256, 0, s>>>(nfwd, fsrc, fcol, d.fval, d.dinv, d.fL);
-    k_ilu_reorg<double><<<grid, 256, 0, s>>>(nbwd, bsrc, bcol, d.fval, d.dinv, d.bU);
+    k_ilu_reorg<double><<<grid, 256, 0, s>>>(nfwd, fsrc, fcol, frow, d.fval, d.dinv, d.fL);
+    k_ilu_reorg<double><<<grid, 256, 0, s>>>(nbwd, bsrc, bcol, brow, d.fval, d.dinv, d.bU);
   }
   count_launch();
   count_launch();
 }
 
-// CTAs of one solve variant that the GPU holds at once (SMs x resident CTAs per SM), found
-// once per variant; 0 if the occupancy query fails (the launch order is then always used)
-template <class T, int CH, int NCW, int RB, bool WIDE>
-int solve_slots() {
-  static const int slots = [] {
-    int dev = 0, nsm = 0, nb = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ilu_solve<T, T, CH, NCW, RB, WIDE>, 32 * (NCW + 1),
-                                                      solve_smem<T>(RB)) != cudaSuccess) {
-      (void)cudaGetLastError();  // the query's own error: nothing was launched
-      return 0;
-    }
-    return nsm * nb;
-  }();
-  return slots;
-}
-
-// The longest-first launch order pays when the subdomain CTAs come in several waves
-// (18.4M nodes, 4096 subdomains: 7.5% off the solve).  When every CTA is resident from
-// the start it only decides which CTAs share an SM, and the natural order measured
-// slightly better (2.0M nodes, 512 subdomains: 2.5%), so a single wave keeps it.
-template <class T, int CH, int NCW, int RB, bool WIDE>
-void launch_ilu_solve_c(const RasDev& d, const double* r, T* z, int32_t* err, cudaStream_t s) {
-  RasDev dl = d;
-  if (d.P <= solve_slots<T, CH, NCW, RB, WIDE>()) dl.sd_sched = nullptr;
-  k_ilu_solve<T, T, CH, NCW, RB, WIDE><<<d.P, 32 * (NCW + 1), solve_smem<T>(RB), s>>>(dl, r, z, err);
-}
-
-// f.template operator()<CH, NCW, RB, WIDE>() for the launch shape of d
-template <class F>
+// f.template operator()<NCW, RB, WIDE>() for the launch shape of d
+template <class T, class F>
 void solve_variant(const RasDev& d, F&& f) {
-  auto ring = [&]<int CH, int NCW, bool WIDE>() {
-    if (d.solve_ring == SOLVE_RING_HALF) f.template operator()<CH, NCW, SOLVE_RING_HALF, WIDE>();
-    else f.template operator()<CH, NCW, SOLVE_RING_FULL, WIDE>();
+  auto warps = [&]<int RB, bool WIDE>() {
+    if (d.solve_warps == 3) f.template operator()<3, RB, WIDE>();
+    else f.template operator()<7, RB, WIDE>();
   };
-  auto warps = [&]<int CH, bool WIDE>() {
-    if (d.solve_warps == 3) ring.template operator()<CH, 3, WIDE>();
-    else ring.template operator()<CH, 7, WIDE>();
+  auto ring = [&]<int A, int B, int C>() {
+    if (d.solve_ring == SOLVE_RING_HALF) warps.template operator()<SOLVE_RING_HALF, false>();
+    else if (d.solve_ring == A) warps.template operator()<A, false>();
+    else if (d.solve_ring == B) warps.template operator()<B, false>();
+    else warps.template operator()<C, false>();
   };
-  auto batch = [&]<bool WIDE>() {
-    switch (d.solve_ch) {
-      case 1: warps.template operator()<1, WIDE>(); break;
-      case 3: warps.template operator()<3, WIDE>(); break;
-      case 4: warps.template operator()<4, WIDE>(); break;
-      default: warps.template operator()<2, WIDE>(); break;
-    }
-  };
-  if (d.P <= SOLVE_WIDE_MAX) batch.template operator()<true>();
-  else batch.template operator()<false>();
+  if (d.P <= SOLVE_WIDE_MAX) {
+    if (d.solve_ring == SOLVE_RING_HALF) warps.template operator()<SOLVE_RING_HALF, true>();
+    else warps.template operator()<SOLVE_RING_1, true>();
+  } else if constexpr (sizeof(T) == 8) {
+    ring.template operator()<SOLVE_RING_2, SOLVE_RING_3, SOLVE_RING_4>();
+  } else {
+    ring.template operator()<SOLVE_RING_2, SOLVE_RING_4F, SOLVE_RING_FULL>();
+  }
 }
 
+// CTAs take the subdomains longest first (sd_sched): with several waves the short ones fill
+// the tail (18.4M nodes, 4096 subdomains: 7.5% off the solve), in one wave it decides which
+// share an SM (1024 x 1024, 512 subdomains: 1.07 -> 1.03 ms in FP64, 0.532 -> 0.525 in FP32).
 template <class T>
-void launch_ilu_solve_t(const RasDev& d, const double* r, T* z, int32_t* err, cudaStream_t s) {
-  solve_variant(d, [&]<int CH, int NCW, int RB, bool WIDE>() {
-    launch_ilu_solve_c<T, CH, NCW, RB, WIDE>(d, r, z, err, s);
+void launch_ilu_solve_t(const RasDev& d, const T* r, T* z, int32_t* err, cudaStream_t s) {
+  solve_variant<T>(d, [&]<int NCW, int RB, bool WIDE>() {
+    k_ilu_solve<T, T, NCW, RB, WIDE><<<d.P, 32 * (solve_consumers(NCW) + 2), solve_smem<T>(RB), s>>>(d, r, z, err);
   });
   count_launch();
 }
@@ -900,29 +891,26 @@ void launch_ilu_solve(const RasDev& d, const double* r, double* z, int32_t* err,
   launch_ilu_solve_t<double>(d, r, z, err, s);
 }
 
-void launch_ilu_solve32(const RasDev& d, const double* r, float* z, int32_t* err, cudaStream_t s) {
+void launch_ilu_solve32(const RasDev& d, const float* r, float* z, int32_t* err, cudaStream_t s) {
   launch_ilu_solve_t<float>(d, r, z, err, s);
 }
 
-// shared-memory limits and resident-CTA counts of every solve variant, set and found here (at
-// context creation) rather than in a captured launch
+// shared-memory limits of every solve variant, set at context creation rather than in a
+// captured launch
 template <class T>
 void solve_attrs_all() {
   RasDev d{};
   for (int P : {1, SOLVE_WIDE_MAX + 1})
     for (int w : {3, 7})
-      for (int rb : {SOLVE_RING_HALF, SOLVE_RING_FULL})
-        for (int ch : {1, 2, 3, 4}) {
-          d.P = P;
-          d.solve_warps = w;
-          d.solve_ring = rb;
-          d.solve_ch = ch;
-          solve_variant(d, []<int CH, int NCW, int RB, bool WIDE>() {
-            cudaFuncSetAttribute(k_ilu_solve<T, T, CH, NCW, RB, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)solve_smem<T>(RB));
-            (void)solve_slots<T, CH, NCW, RB, WIDE>();
-          });
-        }
+      for (int ring : {SOLVE_RING_HALF, SOLVE_RING_1, SOLVE_RING_2, SOLVE_RING_3, SOLVE_RING_4, SOLVE_RING_4F, SOLVE_RING_FULL}) {
+        d.P = P;
+        d.solve_warps = w;
+        d.solve_ring = ring;
+        solve_variant<T>(d, []<int NCW, int RB, bool WIDE>() {
+          cudaFuncSetAttribute(k_ilu_solve<T, T, NCW, RB, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)solve_smem<T>(RB));
+        });
+      }
 }
 
 void launch_coarse_assemble(const CoarseDev& c, const double* val, const float* val32, cudaStream_t s) {
@@ -1038,10 +1026,11 @@ __global__ void k_az_sub(int64_t n, const int64_t* __restrict__ az_ptr, const in
   t[g] -= acc;
 }
 
-// the same with FP32 products for the mixed path (its result feeds an FP32 subdomain solve)
+// the same with FP32 products for the mixed path, whose subdomain solve takes the result in
+// FP32: out = (float)(t - (A Z) y), rows padded to eight values
 __global__ void k_az_sub32(int64_t n, const int64_t* __restrict__ az_ptr, const int32_t* __restrict__ az_unit,
                            const int32_t* __restrict__ cpos, const float* __restrict__ azval,
-                           const float* __restrict__ y, double* __restrict__ t) {
+                           const float* __restrict__ y, const double* __restrict__ t, float* __restrict__ out) {
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= 5 * n) return;
   const int64_t i = g / 5;
@@ -1053,7 +1042,20 @@ __global__ void k_az_sub32(int64_t n, const int64_t* __restrict__ az_ptr, const 
 #pragma unroll
     for (int mm = 0; mm < 5; ++mm) acc = fmaf(A[mm], ys[mm], acc);
   }
-  t[g] -= (double)acc;
+  out[8 * i + rr] = (float)(t[g] - (double)acc);
+}
+
+// r in FP32 for the mixed path's subdomain solve, rows padded to eight values
+__global__ void k_pack32(int64_t n, const double* __restrict__ r, float* __restrict__ out) {
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < 5 * n; g += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = g / 5;
+    out[8 * i + (g - 5 * i)] = (float)r[g];
+  }
+}
+
+void launch_pack32(int64_t n, const double* r, float* out, cudaStream_t s) {
+  k_pack32<<<(unsigned)std::min<int64_t>((5 * n + 255) / 256, 152 * 8), 256, 0, s>>>(n, r, out);
+  count_launch();
 }
 
 void launch_az_build(int64_t nseg, const int32_t* az_blk, const double* val, const float* val32, double* azval,
@@ -1065,11 +1067,15 @@ void launch_az_build(int64_t nseg, const int32_t* az_blk, const double* val, con
 }
 
 void launch_az_sub(const CoarseDev& c, int64_t n, const int64_t* az_ptr, const int32_t* az_unit,
-                   const double* azval, const float* azval32, bool fp32, double* t, cudaStream_t s) {
+                   const double* azval, double* t, cudaStream_t s) {
   const double* y = c.ainvT ? c.crhs + 5 * (int64_t)c.P : c.crhs;
-  const unsigned g = (unsigned)((5 * n + 255) / 256);
-  if (fp32) k_az_sub32<<<g, 256, 0, s>>>(n, az_ptr, az_unit, c.cpos, azval32, c.y32, t);
-  else k_az_sub<double><<<g, 256, 0, s>>>(n, az_ptr, az_unit, c.cpos, azval, y, t);
+  k_az_sub<double><<<(unsigned)((5 * n + 255) / 256), 256, 0, s>>>(n, az_ptr, az_unit, c.cpos, azval, y, t);
+  count_launch();
+}
+
+void launch_az_sub32(const CoarseDev& c, int64_t n, const int64_t* az_ptr, const int32_t* az_unit,
+                     const float* azval, const double* t, float* out, cudaStream_t s) {
+  k_az_sub32<<<(unsigned)((5 * n + 255) / 256), 256, 0, s>>>(n, az_ptr, az_unit, c.cpos, azval, c.y32, t, out);
   count_launch();
 }
 

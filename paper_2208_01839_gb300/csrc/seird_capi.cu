@@ -345,11 +345,7 @@ RasDev ras_dev(seird_ctx* ctx) {
   d.zwork32 = ctx->zwork32;
   auto plan = [](const seird_ctx::PlanPtrs& q) {
     SolvePlanDev s;
-    s.row = q.row;
-    s.start = q.start;
-    s.cnt = q.cnt;
-    s.levpos = q.levpos;
-    s.levblk = q.levblk;
+    s.stage = q.stage;
     s.sd_lev0 = q.sd_lev0;
     s.info = reinterpret_cast<const int4*>(q.info);
     return s;
@@ -361,9 +357,8 @@ RasDev ras_dev(seird_ctx* ctx) {
   d.fL32 = ctx->fL32;
   d.bU32 = ctx->bU32;
   d.wait_polls = ctx->wait_polls;
-  d.solve_ch = ctx->ilu_ch;
   d.solve_warps = ctx->ilu_warps;
-  d.solve_ring = ctx->ilu_ring;
+  d.solve_ring = solve_ring_blocks(ctx->hs.P, ctx->hs.fp32, ctx->ilu_ring == SOLVE_RING_HALF, ctx->hs.max_row_blocks);
   return d;
 }
 
@@ -398,7 +393,7 @@ int pc_setup(seird_ctx* ctx) {
     const RasDev d = ras_dev(ctx);
     launch_ilu_factor(d, ctx->val, ctx->val32, ctx->err, mixed(ctx), ctx->stream);
     launch_ilu_reorg(d, (int64_t)ctx->hs.sp_fwd.src.size(), (int64_t)ctx->hs.sp_bwd.src.size(), ctx->pf.src,
-                     ctx->pf.col, ctx->pb.src, ctx->pb.col, mixed(ctx), ctx->stream);
+                     ctx->pf.col, ctx->pf.brow, ctx->pb.src, ctx->pb.col, ctx->pb.brow, mixed(ctx), ctx->stream);
   }
   CK(cudaGetLastError());
   if (ctx->opt.coarse) {
@@ -454,13 +449,12 @@ int pc_apply32(seird_ctx* ctx, const double* r, float* z) {
       add_bytes(ctx, SEIRD_K_COARSE_APPLY, bytes_coarse_solve(ctx) + 80.0 * ctx->hs.n + bytes_az_sub(ctx, 4.0));
       launch_coarse_solve(cd, r, ctx->stream);
       launch_coarse_y32(cd, ctx->stream);
-      CK(cudaMemcpyAsync(ctx->pct, r, sizeof(double) * len, cudaMemcpyDeviceToDevice, ctx->stream));
-      launch_az_sub(cd, ctx->hs.n, ctx->az_ptr, ctx->az_unit, ctx->azval, ctx->azval32, true, ctx->pct, ctx->stream);
+      launch_az_sub32(cd, ctx->hs.n, ctx->az_ptr, ctx->az_unit, ctx->azval32, r, ctx->pcr32, ctx->stream);
     }
     {
       KTimer kt_(ctx, SEIRD_K_ILU_SOLVE);
       add_bytes(ctx, SEIRD_K_ILU_SOLVE, bytes_ilu_solve(ctx, 4.0));
-      launch_ilu_solve32(ras_dev(ctx), ctx->pct, z, ctx->err, ctx->stream);
+      launch_ilu_solve32(ras_dev(ctx), ctx->pcr32, z, ctx->err, ctx->stream);
     }
     {
       KTimer kt_(ctx, SEIRD_K_COARSE_APPLY);
@@ -473,7 +467,8 @@ int pc_apply32(seird_ctx* ctx, const double* r, float* z) {
   {
     KTimer kt_(ctx, SEIRD_K_ILU_SOLVE);
     add_bytes(ctx, SEIRD_K_ILU_SOLVE, bytes_ilu_solve(ctx, 4.0));
-    launch_ilu_solve32(ras_dev(ctx), r, z, ctx->err, ctx->stream);
+    launch_pack32(ctx->hs.n, r, ctx->pcr32, ctx->stream);
+    launch_ilu_solve32(ras_dev(ctx), ctx->pcr32, z, ctx->err, ctx->stream);
   }
   if (ctx->opt.coarse == 1) {
     KTimer kt_(ctx, SEIRD_K_COARSE_APPLY);
@@ -493,12 +488,12 @@ int pc_apply32(seird_ctx* ctx, const double* r, float* z) {
       launch_coarse_y32(cd, ctx->stream);
       launch_coarse_prolong32(cd, ctx->hs.n, z, ctx->stream);
       // r - J (z + Z y) = (r - J z) - (J Z) y, with J Z summed at set-up
-      launch_az_sub(cd, ctx->hs.n, ctx->az_ptr, ctx->az_unit, ctx->azval, ctx->azval32, true, ctx->pct, ctx->stream);
+      launch_az_sub32(cd, ctx->hs.n, ctx->az_ptr, ctx->az_unit, ctx->azval32, ctx->pct, ctx->pcr32, ctx->stream);
     }
     {
       KTimer kt_(ctx, SEIRD_K_ILU_SOLVE);
       add_bytes(ctx, SEIRD_K_ILU_SOLVE, bytes_ilu_solve(ctx, 4.0));
-      launch_ilu_solve32(ras_dev(ctx), ctx->pct, ctx->pcu32, ctx->err, ctx->stream);
+      launch_ilu_solve32(ras_dev(ctx), ctx->pcr32, ctx->pcu32, ctx->err, ctx->stream);
     }
     launch_add32(len, ctx->pcu32, z, ctx->stream);
   }
@@ -524,7 +519,7 @@ int pc_apply(seird_ctx* ctx, const double* r, double* z) {
       add_bytes(ctx, SEIRD_K_COARSE_APPLY, bytes_coarse_solve(ctx) + 80.0 * ctx->hs.n + bytes_az_sub(ctx, 8.0));
       launch_coarse_solve(cd, r, ctx->stream);
       CK(cudaMemcpyAsync(ctx->pct, r, sizeof(double) * len, cudaMemcpyDeviceToDevice, ctx->stream));
-      launch_az_sub(cd, ctx->hs.n, ctx->az_ptr, ctx->az_unit, ctx->azval, ctx->azval32, false, ctx->pct, ctx->stream);
+      launch_az_sub(cd, ctx->hs.n, ctx->az_ptr, ctx->az_unit, ctx->azval, ctx->pct, ctx->stream);
     }
     {
       KTimer kt_(ctx, SEIRD_K_ILU_SOLVE);
@@ -558,7 +553,7 @@ int pc_apply(seird_ctx* ctx, const double* r, double* z) {
       const CoarseDev cd = coarse_dev(ctx);
       launch_coarse_apply_add<double>(cd, ctx->hs.n, ctx->pct, z, ctx->stream);
       // r - J (z + Z y) = (r - J z) - (J Z) y, with J Z summed at set-up
-      launch_az_sub(cd, ctx->hs.n, ctx->az_ptr, ctx->az_unit, ctx->azval, ctx->azval32, false, ctx->pct, ctx->stream);
+      launch_az_sub(cd, ctx->hs.n, ctx->az_ptr, ctx->az_unit, ctx->azval, ctx->pct, ctx->stream);
     }
     {
       KTimer kt_(ctx, SEIRD_K_ILU_SOLVE);
@@ -623,11 +618,6 @@ int norm2(seird_ctx* ctx, const double* x, double* out) {
 // *converged = false (Newton then takes the inexact step).
 bool verbose();
 
-// Largest stage of the solve plans in blocks (a stage has to fit the factor ring).
-int64_t solve_max_stage_blocks(const seird_ctx* ctx) {
-  return std::max<int64_t>(ctx->hs.sp_fwd.max_lev_blocks, ctx->hs.sp_bwd.max_lev_blocks);
-}
-
 // Launch-shape autotuner (options.autotune): times the candidates on the context's own
 // vectors (V[0] holds the first Krylov vector; the Gram-Schmidt candidates run at depth 8
 // with V[1..7] set to copies of it, which GMRES overwrites later) and keeps the fastest.
@@ -652,7 +642,6 @@ int autotune(seird_ctx* ctx) {
     return best;
   };
   float tbest = 1e30f;
-  int best_ch = 0;
   for (int tb : {128, 256, 512}) {
     const float t = best_of([&] {
       if (mixed(ctx)) launch_spmv32(ctx->hs.n, ctx->row_ptr, ctx->col, ctx->val32, ctx->Z32, ctx->tune_buf, s, tb);
@@ -682,36 +671,32 @@ int autotune(seird_ctx* ctx) {
       }
     }
   }
-  // subdomain solves: the dependency-load batch and the consumer warps per CTA, on the
-  // context's own factors with V[0] as the right-hand side (every choice forms the same
-  // sums; only the time differs)
+  // subdomain solves: the shape of their CTAs and of the factor ring, on the context's own
+  // factors with V[0] as the right-hand side (every choice forms the same sums; only the
+  // time differs)
   if (ctx->pc_ready) {
     tbest = 1e30f;
-    const int keep_ch = ctx->ilu_ch, keep_w = ctx->ilu_warps, keep_r = ctx->ilu_ring;
+    if (mixed(ctx)) launch_pack32(ctx->hs.n, ctx->V, ctx->pcr32, s);
+    const int keep_w = ctx->ilu_warps, keep_r = ctx->ilu_ring;
     int best_w = 0, best_r = 0;
-    const bool half_ok = solve_max_stage_blocks(ctx) <= SOLVE_RING_HALF;
+    const bool half_ok = ctx->hs.max_row_blocks <= SOLVE_RING_HALF;
     for (int ring : {SOLVE_RING_FULL, SOLVE_RING_HALF}) {
       if (ring == SOLVE_RING_HALF && !half_ok) continue;
       for (int nw : {7, 3}) {
-        for (int ch : {1, 2, 3, 4}) {
-          ctx->ilu_ch = ch;
-          ctx->ilu_warps = nw;
-          ctx->ilu_ring = ring;
-          const RasDev d = ras_dev(ctx);
-          const float t = best_of([&] {
-            if (mixed(ctx)) launch_ilu_solve32(d, ctx->V, reinterpret_cast<float*>(ctx->tune_buf), ctx->err, s);
-            else launch_ilu_solve(d, ctx->V, ctx->tune_buf, ctx->err, s);
-          });
-          if (t < tbest) {
-            tbest = t;
-            best_ch = ch;
-            best_w = nw;
-            best_r = ring;
-          }
+        ctx->ilu_warps = nw;
+        ctx->ilu_ring = ring;
+        const RasDev d = ras_dev(ctx);
+        const float t = best_of([&] {
+          if (mixed(ctx)) launch_ilu_solve32(d, ctx->pcr32, reinterpret_cast<float*>(ctx->tune_buf), ctx->err, s);
+          else launch_ilu_solve(d, ctx->V, ctx->tune_buf, ctx->err, s);
+        });
+        if (t < tbest) {
+          tbest = t;
+          best_w = nw;
+          best_r = ring;
         }
       }
     }
-    ctx->ilu_ch = best_ch > 0 ? best_ch : keep_ch;
     ctx->ilu_warps = best_w > 0 ? best_w : keep_w;
     ctx->ilu_ring = best_r > 0 ? best_r : keep_r;
   }
@@ -719,8 +704,8 @@ int autotune(seird_ctx* ctx) {
   cudaEventDestroy(e1);
   CK(cudaGetLastError());
   if (verbose())
-    std::fprintf(stderr, "[seird] autotune: spmv %d threads, gram-schmidt %d CTAs, tile %d, ilu batch %d warps %d "
-                 "ring %d\n", ctx->spmv_tb, ctx->red_grid, ctx->cgs_tile, ctx->ilu_ch, ctx->ilu_warps, ctx->ilu_ring);
+    std::fprintf(stderr, "[seird] autotune: spmv %d threads, gram-schmidt %d CTAs, tile %d, ilu warps %d ring %d\n",
+                 ctx->spmv_tb, ctx->red_grid, ctx->cgs_tile, ctx->ilu_warps, ctx->ilu_ring);
   return SEIRD_OK;
 }
 
@@ -1476,7 +1461,7 @@ static int create_impl(seird_ctx* ctx, const seird_mesh* mesh, const seird_param
     return fail(ctx, SEIRD_EINVAL, "coarse space supports at most 5120 coarse units (options.coarse_group)");
   // a stage of the subdomain solves must fit the factor ring (only a row with more blocks than
   // the ring, a node with hundreds of neighbours, can make one larger)
-  if (solve_max_stage_blocks(ctx) > SOLVE_RING_FULL)
+  if (hs.max_row_blocks > SOLVE_RING_FULL)
     return fail(ctx, SEIRD_EINVAL, "a subdomain row has more blocks than the solve's shared-memory ring holds (" +
                                        std::to_string(SOLVE_RING_FULL) + ")");
   if (o.stream) {
@@ -1578,11 +1563,8 @@ static int create_impl(seird_ctx* ctx, const seird_mesh* mesh, const seird_param
   for (int dir = 0; dir < 2; ++dir) {
     const HostSetup::SolvePlan& sp = dir == 0 ? hs.sp_fwd : hs.sp_bwd;
     seird_ctx::PlanPtrs& q = dir == 0 ? ctx->pf : ctx->pb;
-    TRY(upload(ctx, &q.row, sp.row));
-    TRY(upload(ctx, &q.start, sp.start));
-    TRY(upload(ctx, &q.cnt, sp.cnt));
-    TRY(upload(ctx, &q.levpos, sp.levpos));
-    TRY(upload(ctx, &q.levblk, sp.levblk));
+    TRY(upload(ctx, &q.stage, sp.stage));
+    TRY(upload(ctx, &q.brow, sp.brow));
     TRY(upload(ctx, &q.sd_lev0, sp.sd_lev0));
     TRY(upload(ctx, &q.src, sp.src));
     TRY(upload(ctx, &q.col, sp.col));
@@ -1591,15 +1573,16 @@ static int create_impl(seird_ctx* ctx, const seird_mesh* mesh, const seird_param
     else TRY(dalloc(ctx, dir == 0 ? &ctx->fL : &ctx->bU, (size_t)26 * std::max<size_t>(1, sp.src.size())));
   }
   if (mix) {
+    TRY(dalloc(ctx, &ctx->pcr32, 8 * (size_t)n));
     TRY(dalloc(ctx, &ctx->fval32, 25 * NLB));
     TRY(dalloc(ctx, &ctx->dinv32, 25 * NL));
-    TRY(dalloc(ctx, &ctx->ywork32, 5 * NL));
-    TRY(dalloc(ctx, &ctx->zwork32, 5 * NL));
+    TRY(dalloc(ctx, &ctx->ywork32, SOLVE_STRIDE<float> * NL));
+    TRY(dalloc(ctx, &ctx->zwork32, SOLVE_STRIDE<float> * NL));
   } else {
     TRY(dalloc(ctx, &ctx->fval, 25 * NLB));
     TRY(dalloc(ctx, &ctx->dinv, 25 * NL));
-    TRY(dalloc(ctx, &ctx->ywork, 5 * NL));
-    TRY(dalloc(ctx, &ctx->zwork, 5 * NL));
+    TRY(dalloc(ctx, &ctx->ywork, SOLVE_STRIDE<double> * NL));
+    TRY(dalloc(ctx, &ctx->zwork, SOLVE_STRIDE<double> * NL));
   }
   // coarse
   if (o.coarse >= 2) {
@@ -1944,7 +1927,7 @@ int seird_set_launch_shapes(seird_ctx* ctx, int32_t spmv_threads, int32_t cgs_ct
       ilu_batch > 4 || (ilu_warps && ilu_warps != 3 && ilu_warps != 7) ||
       (ilu_ring && ilu_ring != SOLVE_RING_FULL && ilu_ring != SOLVE_RING_HALF))
     return fail(ctx, SEIRD_EINVAL, "set_launch_shapes: a shape outside its candidates");
-  if (ilu_ring == SOLVE_RING_HALF && solve_max_stage_blocks(ctx) > SOLVE_RING_HALF)
+  if (ilu_ring == SOLVE_RING_HALF && ctx->hs.max_row_blocks > SOLVE_RING_HALF)
     return fail(ctx, SEIRD_EINVAL, "set_launch_shapes: a solve stage is larger than a one-stage ring");
   if (ilu_ring) ctx->ilu_ring = ilu_ring;
   if (spmv_threads) ctx->spmv_tb = spmv_threads;

@@ -238,6 +238,48 @@ static void iluk_pattern(int k, int32_t nl, std::vector<int64_t>& rstart, std::v
   for (int32_t i = 0; i < nl; ++i) rstart[i + 1] = rowend[i];
 }
 
+// Where the solve's copies of each stage of subdomain q go in shared memory, and which stage
+// must have been consumed before them.  The rings fill in stage order (forward, then
+// backward sweep) and a stage does not wrap around a ring's end, so all of it is known
+// here: the row ring and, for both sizes of the factor ring, the block ring offset and the
+// distance back to the last stage that is in the way (SOLVE_FREE: none).  The first backward
+// stage waits for the whole forward sweep, whose results it reads.
+static void place_stages(HostSetup& hs, int32_t q) {
+  const int32_t nF = hs.sp_fwd.sd_lev0[q + 1] - hs.sp_fwd.sd_lev0[q] - 1;
+  const int32_t nB = hs.sp_bwd.sd_lev0[q + 1] - hs.sp_bwd.sd_lev0[q] - 1;
+  auto rec = [&](int32_t g) {
+    return g < nF ? &hs.sp_fwd.stage[hs.sp_fwd.sd_lev0[q] + g] : &hs.sp_bwd.stage[hs.sp_bwd.sd_lev0[q] + g - nF];
+  };
+  constexpr int32_t NS = SOLVE_SLOTS;
+  int64_t vr[2] = {0, 0}, vb[2] = {0, 0}, start_r[2][NS], start_b[2][NS];
+  const int32_t ring[2] = {solve_ring_blocks(hs.P, hs.fp32, false, hs.max_row_blocks) + SOLVE_RING_SPARE,
+                           solve_ring_blocks(hs.P, hs.fp32, true, hs.max_row_blocks) + SOLVE_RING_SPARE};
+  auto place = [](int64_t head, int32_t count, int32_t size) {
+    return head % size + count > size ? head + size - head % size : head;
+  };
+  for (int32_t g = 0; g < nF + nB; ++g) {
+    int4* st = rec(g);
+    const int32_t nr = stage_rows(*st), nb = stage_blocks(*st);
+    uint32_t w = 0, wr = 0;
+    for (int v = 0; v < 2; ++v) {
+      const int64_t sr = place(vr[v], nr, solve_ring_rows(ring[v] - SOLVE_RING_SPARE));
+      const int64_t sb = place(vb[v], nb, ring[v]);
+      int32_t need = g == nF ? g - 1 : g - NS;
+      for (int32_t o = g - 1; o > need && o > g - NS; --o)
+        if (sr + nr - start_r[v][o % NS] > solve_ring_rows(ring[v] - SOLVE_RING_SPARE) || sb + nb - start_b[v][o % NS] > ring[v]) need = o;
+      const int32_t dist = need < 0 ? SOLVE_FREE : g - need;
+      w |= ((uint32_t)(sb % ring[v]) | (uint32_t)dist << 10) << (16 * v);
+      start_b[v][g % NS] = sb;
+      start_r[v][g % NS] = sr;
+      vb[v] = sb + nb;
+      vr[v] = sr + nr;
+      wr |= (uint32_t)(sr % solve_ring_rows(ring[v] - SOLVE_RING_SPARE)) << (8 * v);
+    }
+    st->z |= (int32_t)(wr << 16);
+    st->w = (int32_t)w;
+  }
+}
+
 int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs, std::string& err) {
   const int64_t n = mesh->n_nodes, m = mesh->n_tris;
   if (n < 3 || m < 1 || !mesh->xy || !mesh->tri) {
@@ -278,6 +320,7 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
     return SEIRD_EINVAL;
   }
   hs.ilu_fill = opt->ilu_fill;
+  hs.fp32 = opt->precision == 1;
 
   // ---- internal numbering: nodes sorted by (owner, caller index) ----------
   hs.own_ptr.assign(P + 1, 0);
@@ -473,7 +516,7 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
         for (int64_t a = rstart[i]; a < rstart[i + 1]; ++a) rowpos[S.l_col[a]] = -1;
       }
       // forward levels (lower triangle) and backward levels (upper triangle)
-      std::vector<int32_t> lev(nl);
+      std::vector<int32_t> lev(nl), cnt(nl);
       for (int dir = 0; dir < 2; ++dir) {
         int32_t nlev = 0;
         if (dir == 0) {
@@ -505,6 +548,13 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
         } else {
           for (int32_t i = nl - 1; i >= 0; --i) order[fill[lev[i]]++] = i;
         }
+        // the rows of a level are independent: longest first, so that rows of about the same
+        // length share a warp in the factorisation and the solves
+        for (int32_t i = 0; i < nl; ++i)
+          cnt[i] = (int32_t)(dir == 0 ? S.diag[i] - rstart[i] : rstart[i + 1] - S.diag[i] - 1);
+        for (int32_t v = 0; v < nlev; ++v)
+          std::stable_sort(order.begin() + lb[v], order.begin() + lb[v + 1],
+                           [&](int32_t a, int32_t b) { return cnt[a] > cnt[b]; });
       }
       for (int32_t l = 0; l < nl; ++l) loc[nodes[l]] = -1;
     });
@@ -583,18 +633,23 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
     parts.shrink_to_fit();
   }
 
-  // ---- ILU(0) solve plans ---------------------------------------------------
-  // The solve numbers a subdomain's solution entries by their position in the
-  // sweep (forward y and backward z each in their own order), so the column of
-  // every factor block is the position of the entry it multiplies, and a row
-  // record holds: forward (node, first block, block count, 0); backward (forward
-  // position of the row, first block, block count, node if the subdomain owns it
+  // ---- ILU solve plans --------------------------------------------------------
+  // The sweeps run on the factors scaled by the inverted pivots (k_ilu_reorg), so that
+  // a row's result is one sum of block products and no step follows it:
+  //   forward   y_i = Dinv_i r_i - sum_j (Dinv_i L_ij U_jj) y_j
+  //   backward  z_i = y_i - sum_j (Dinv_i U_ij) z_j.
+  // Forward rows hold Dinv_i first (no column), then the strictly lower blocks; backward rows hold the
+  // strictly upper ones.  The solve numbers a subdomain's solution entries by their
+  // position in the sweep (forward y and backward z each in their own order), so the
+  // column of a factor block is the position of the entry it multiplies, as -1 - position
+  // where the entry has left the solve's window (SOLVE_WIN) by then, and a row record holds: forward (node, first block, block count, position in the backward sweep);
+  // backward (forward position, first block, block count, node if the subdomain owns it
   // else -1).
   // Built per subdomain in parallel (block indices relative to the subdomain's first
   // solve block), then concatenated in subdomain order.
   struct PlanPart {
-    std::vector<int32_t> levpos, row, cnt, info, col;
-    std::vector<int64_t> levblk, start, src;
+    std::vector<int32_t> levpos, info, col, brow;
+    std::vector<int64_t> levblk, src;
   };
   for (int dir = 0; dir < 2; ++dir) {
     HostSetup::SolvePlan& sp = dir == 0 ? hs.sp_fwd : hs.sp_bwd;
@@ -606,10 +661,10 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
       PlanPart& T = pp[q];
       const int32_t r0 = hs.sd_row0[q];
       const int32_t nlq = hs.sd_row0[q + 1] - r0;
-      std::vector<int32_t> posf(nlq, 0), posd(nlq, 0);
+      std::vector<int32_t> posf(nlq, 0), posb(nlq, 0);
       for (int32_t k = 0; k < nlq; ++k) {
         posf[hs.fwd_order[r0 + k]] = k;
-        posd[order[r0 + k]] = k;
+        posb[hs.bwd_order[r0 + k]] = k;
       }
       const int32_t nlev = lev0[q + 1] - lev0[q] - 1;
       T.levpos.push_back(0);
@@ -619,40 +674,33 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
         for (int32_t k = levs[lev0[q] + v]; k < levs[lev0[q] + v + 1]; ++k) {
           const int32_t i = order[r0 + k];
           const int64_t R = (int64_t)r0 + i;
-          int32_t nb = 0;
-          if (dir == 0) {
-            nb = (int32_t)(hs.l_diag[R] - hs.l_row_ptr[R]);
-          } else {
-            nb = 1 + (int32_t)(hs.l_row_ptr[R + 1] - hs.l_diag[R] - 1);
-          }
-          if ((in_level > 0 && in_level + nb > SOLVE_BUF_BLOCKS) ||
+          const int32_t nb = (int32_t)(dir == 0 ? 1 + hs.l_diag[R] - hs.l_row_ptr[R] : hs.l_row_ptr[R + 1] - hs.l_diag[R] - 1);
+          if ((pos > T.levpos.back() && in_level + nb > SOLVE_BUF_BLOCKS) ||
               pos - T.levpos.back() >= SOLVE_BUF_ROWS) {  // split: rows of a level are independent
             T.levpos.push_back(pos);
             T.levblk.push_back((int64_t)T.src.size());
             in_level = 0;
           }
-          T.row.push_back(i);
-          T.start.push_back((int64_t)T.src.size());
-          T.cnt.push_back(nb);
           const int32_t node = hs.sd_node[R];
           const bool owned = node >= hs.own_ptr[q] && node < hs.own_ptr[q + 1];
           T.info.push_back(dir == 0 ? node : posf[i]);
           T.info.push_back((int32_t)((int64_t)T.src.size() - T.levblk.back()));
           T.info.push_back(nb);
-          T.info.push_back(dir == 0 ? 0 : (owned ? node : -1));
+          T.info.push_back(dir == 0 ? posb[i] : (owned ? node : -1));
           if (dir == 0) {
+            T.src.push_back(-1 - R);
+            T.col.push_back(0);
             for (int64_t a = hs.l_row_ptr[R]; a < hs.l_diag[R]; ++a) {
               T.src.push_back(a);
               T.col.push_back(posf[hs.l_col[a]]);
             }
           } else {
-            T.src.push_back(-1 - R);
-            T.col.push_back(posd[i]);
             for (int64_t a = hs.l_diag[R] + 1; a < hs.l_row_ptr[R + 1]; ++a) {
               T.src.push_back(a);
-              T.col.push_back(posd[hs.l_col[a]]);
+              T.col.push_back(posb[hs.l_col[a]]);
             }
           }
+          T.brow.resize(T.src.size(), (int32_t)R);
           in_level += nb;
           ++pos;
         }
@@ -662,39 +710,43 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
       }
     });
     // concatenation: slices from prefix sums, copied in parallel
-    std::vector<int64_t> loff(P + 1, 0), roff(P + 1, 0), soff(P + 1, 0);
+    std::vector<int64_t> loff(P + 1, 0), soff(P + 1, 0);
     for (int32_t q = 0; q < P; ++q) {
       loff[q + 1] = loff[q] + (int64_t)pp[q].levpos.size();
-      roff[q + 1] = roff[q] + (int64_t)pp[q].row.size();
       soff[q + 1] = soff[q] + (int64_t)pp[q].src.size();
     }
     sp.sd_lev0.resize(P + 1);
     for (int32_t q = 0; q <= P; ++q) sp.sd_lev0[q] = (int32_t)loff[q];
     sp.levpos.resize(loff[P]);
     sp.levblk.resize(loff[P]);
-    sp.row.resize(roff[P]);
-    sp.start.resize(roff[P]);
-    sp.cnt.resize(roff[P]);
-    sp.info.resize(4 * roff[P]);
+    sp.stage.assign(loff[P], make_int4(0, 0, 0, 0));
+    sp.info.resize(4 * (size_t)hs.sd_row0[P]);
     sp.src.resize(soff[P]);
     sp.col.resize(soff[P]);
+    sp.brow.resize(soff[P]);
     parallel_for(P, setup_threads(P), [&](int32_t q, int) {
       PlanPart& T = pp[q];
-      const int64_t l0 = loff[q], r0 = roff[q], s0 = soff[q];
+      const int64_t l0 = loff[q], r0 = hs.sd_row0[q], s0 = soff[q];
       std::copy(T.levpos.begin(), T.levpos.end(), sp.levpos.begin() + l0);
       for (size_t k = 0; k < T.levblk.size(); ++k) sp.levblk[l0 + k] = s0 + T.levblk[k];
-      std::copy(T.row.begin(), T.row.end(), sp.row.begin() + r0);
-      for (size_t k = 0; k < T.start.size(); ++k) sp.start[r0 + k] = s0 + T.start[k];
-      std::copy(T.cnt.begin(), T.cnt.end(), sp.cnt.begin() + r0);
       std::copy(T.info.begin(), T.info.end(), sp.info.begin() + 4 * r0);
       std::copy(T.src.begin(), T.src.end(), sp.src.begin() + s0);
       std::copy(T.col.begin(), T.col.end(), sp.col.begin() + s0);
+      std::copy(T.brow.begin(), T.brow.end(), sp.brow.begin() + s0);
+      for (size_t v = 0; v + 1 < T.levpos.size(); ++v) {
+        const int32_t q0 = T.levpos[v], nr = T.levpos[v + 1] - q0;
+        // entries that this stage's results displace from the window, and older ones
+        for (int64_t a = s0 + T.levblk[v]; a < s0 + T.levblk[v + 1]; ++a)
+          if (sp.src[a] >= 0 && sp.col[a] < q0 + nr - SOLVE_WIN) sp.col[a] = -1 - sp.col[a];
+        sp.stage[l0 + v] = make_int4(q0, (int32_t)(s0 + T.levblk[v]), nr | (int32_t)(T.levblk[v + 1] - T.levblk[v]) << 8, 0);
+      }
       T = PlanPart();
     });
-    for (int32_t q = 0; q < P; ++q)
-      for (int32_t v = sp.sd_lev0[q]; v + 1 < sp.sd_lev0[q + 1]; ++v)
-        sp.max_lev_blocks = std::max<int32_t>(sp.max_lev_blocks, (int32_t)(sp.levblk[v + 1] - sp.levblk[v]));
   }
+  for (size_t R = 0; R < hs.l_diag.size(); ++R)
+    hs.max_row_blocks = std::max<int64_t>({hs.max_row_blocks, hs.l_diag[R] - hs.l_row_ptr[R],
+                                           hs.l_row_ptr[R + 1] - hs.l_diag[R]});
+  parallel_for(P, setup_threads(P), [&](int32_t q, int) { place_stages(hs, q); });
 
   // ---- launch order of the subdomain CTAs ------------------------------------
   // Subdomains differ in size (2k-8k nodes at 4096 subdomains) and several waves of
@@ -931,11 +983,10 @@ int64_t check_setup(const HostSetup& hs, std::string& first) {
     const std::vector<int32_t>& order = dir == 0 ? hs.fwd_order : hs.bwd_order;
     for (int32_t q = 0; q < P && !bad; ++q) {
       const int32_t r0 = hs.sd_row0[q], nl = hs.sd_row0[q + 1] - r0;
-      std::vector<int32_t> posf(nl, -1), hit(nl, 0);
+      std::vector<int32_t> hit(nl, 0);
       for (int32_t k = 0; k < nl; ++k) {
         const int32_t i = order[r0 + k];
         fail(i >= 0 && i < nl && hit[i]++ == 0, "sweep order is not a permutation");
-        if (i >= 0 && i < nl) posf[i] = k;
       }
       const int32_t v0 = sp.sd_lev0[q], v1 = sp.sd_lev0[q + 1] - 1;
       fail(sp.levpos[v0] == 0 && sp.levpos[v1] == nl, "stage positions");
@@ -943,7 +994,11 @@ int64_t check_setup(const HostSetup& hs, std::string& first) {
       for (int32_t v = v0; v < v1 && !bad; ++v) {
         const int32_t k0 = sp.levpos[v], k1 = sp.levpos[v + 1];
         const int64_t b0 = sp.levblk[v], nbs = sp.levblk[v + 1] - b0;
-        fail(k1 >= k0 && k1 - k0 <= SOLVE_BUF_ROWS && nbs >= 0 && nbs <= SOLVE_BUF_BLOCKS, "stage exceeds the rings");
+        // (a forward row holds its inverted pivot besides its lower blocks)
+        fail(k1 >= k0 && k1 - k0 <= SOLVE_BUF_ROWS && nbs >= 0 && nbs <= SOLVE_BUF_BLOCKS + (dir == 0 && k1 - k0 == 1),
+             "stage exceeds the rings");
+        const int4 st = sp.stage[v];
+        fail(st.x == k0 && st.y == b0 && stage_rows(st) == k1 - k0 && stage_blocks(st) == nbs, "stage record");
         for (int32_t k = k0; k < k1; ++k) {
           const int32_t* rec = &sp.info[4 * ((int64_t)r0 + k)];
           const int32_t i = order[r0 + k];
@@ -951,26 +1006,51 @@ int64_t check_setup(const HostSetup& hs, std::string& first) {
           fail(rec[1] >= 0 && rec[2] >= 0 && rec[1] + rec[2] <= nbs, "row record outside its stage");
           int32_t expect = 0;
           if (dir == 0) {
-            for (int64_t a = hs.l_row_ptr[R]; a < hs.l_diag[R]; ++a) ++expect;
-            fail(rec[0] == hs.sd_node[R] && rec[3] == 0, "forward record");
+            expect = 1 + (int32_t)(hs.l_diag[R] - hs.l_row_ptr[R]);
+            fail(rec[0] == hs.sd_node[R] && rec[3] >= 0 && rec[3] < nl && hs.bwd_order[r0 + rec[3]] == i, "forward record");
+            fail(sp.src[b0 + rec[1]] == -1 - R, "forward pivot block");
           } else {
-            expect = 1 + (int32_t)(hs.l_row_ptr[R + 1] - hs.l_diag[R] - 1);
+            expect = (int32_t)(hs.l_row_ptr[R + 1] - hs.l_diag[R] - 1);
             const int32_t node = hs.sd_node[R];
             const bool own = node >= hs.own_ptr[q] && node < hs.own_ptr[q + 1];
             fail(rec[0] >= 0 && rec[0] < nl && hs.fwd_order[r0 + rec[0]] == i, "backward record: forward position");
             fail(rec[3] == (own ? node : -1), "backward record: owned node");
             owned += own;
-            fail(sp.src[b0 + rec[1]] == -1 - R && sp.col[b0 + rec[1]] == k, "backward pivot block");
           }
           fail(rec[2] == expect, "row block count");
-          for (int32_t j = dir == 0 ? 0 : 1; j < rec[2]; ++j) {
-            const int32_t pos = sp.col[b0 + rec[1] + j];
+          for (int32_t j = 0; j < rec[2]; ++j) fail(sp.brow[b0 + rec[1] + j] == R, "factor block of another row");
+          for (int32_t j = dir == 0 ? 1 : 0; j < rec[2]; ++j) {
+            const int32_t c = sp.col[b0 + rec[1] + j], pos = c < 0 ? -1 - c : c;
             fail(pos >= 0 && pos < k0, "dependency not in an earlier stage");
+            fail((c < 0) == (pos < k1 - SOLVE_WIN), "dependency's place (window or work array)");
           }
         }
       }
       if (dir == 1) fail(owned == hs.own_ptr[q + 1] - hs.own_ptr[q], "owned rows written once");
     }
+  }
+  // ring placement: no stage overlaps one that need not have been consumed before it
+  for (int32_t q = 0; q < P && !bad && hs.max_row_blocks <= SOLVE_RING_HALF; ++q) {
+    const int32_t f0 = hs.sp_fwd.sd_lev0[q], nF = hs.sp_fwd.sd_lev0[q + 1] - f0 - 1;
+    const int32_t l0 = hs.sp_bwd.sd_lev0[q], ng = nF + hs.sp_bwd.sd_lev0[q + 1] - l0 - 1;
+    auto rec = [&](int32_t g) { return g < nF ? hs.sp_fwd.stage[f0 + g] : hs.sp_bwd.stage[l0 + g - nF]; };
+    for (int v = 0; v < 2; ++v)
+      for (int32_t g = 0, free_to = -1; g < ng && !bad; ++g) {  // stages up to free_to have been consumed
+        const int4 st = rec(g);
+        const int32_t dist = stage_distance(st, v), blocks = solve_ring_blocks(P, hs.fp32, v == 1, hs.max_row_blocks);
+        if (dist != SOLVE_FREE) free_to = std::max(free_to, g - dist);
+        fail(dist >= 1 && (dist <= SOLVE_SLOTS || dist == SOLVE_FREE) && g - free_to <= SOLVE_SLOTS, "stage slot reused");
+        fail(g != nF || free_to == g - 1, "backward sweep starts early");
+        const int32_t rb = stage_block_offset(st, v), rr = stage_row_offset(st, v);
+        fail(rb + stage_blocks(st) <= blocks + SOLVE_RING_SPARE && rr + stage_rows(st) <= solve_ring_rows(blocks),
+             "stage wraps around a ring");
+        for (int32_t o = std::max(0, free_to + 1); o < g; ++o) {
+          const int4 so = rec(o);
+          const int32_t ob = stage_block_offset(so, v), orr = stage_row_offset(so, v);
+          fail(rb >= ob + stage_blocks(so) || ob >= rb + stage_blocks(st), "stages overlap in the factor ring");
+          fail(rr >= orr + stage_rows(so) || orr >= rr + stage_rows(st), "stages overlap in the row ring");
+        }
+      }
   }
   // launch order: every subdomain once (each CTA writes only the nodes its subdomain
   // owns), longest first
