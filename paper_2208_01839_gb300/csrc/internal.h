@@ -63,8 +63,12 @@ struct HostSetup {
   std::vector<int32_t> l_col;       // [NLB] local column (row index within the subdomain)
   std::vector<int32_t> l_gblk;      // [NLB] global J block of each local block
   std::vector<int64_t> l_diag;      // [NL] absolute index of the diagonal block
-  std::vector<int64_t> upd_ptr;     // [NLB+1] ILU(0) update pairs of each lower block
-  std::vector<int64_t> upd;         // [2*nupd] (destination block, source block) pairs
+  std::vector<int64_t> upd_ptr;     // [NLB+1] update pairs of each lower block
+  std::vector<int32_t> upd;         // [2*nupd] pairs (destination | lower block << 16, both within the row; source block)
+  // the factorisation's row records in forward order: row, first block, blocks | lower blocks << 16,
+  // pairs; and the row's first pair
+  std::vector<int4> frec;           // [NL]
+  std::vector<int64_t> fpair;       // [NL]
   std::vector<int32_t> fwd_order;   // [NL] local rows (relative) grouped by forward level
   std::vector<int32_t> fwd_lev;     // level boundaries (relative to the subdomain's rows)
   std::vector<int32_t> sd_fwd_lev0; // [P+1] offsets into fwd_lev (each subdomain has nlev+1 entries)
@@ -213,18 +217,12 @@ struct seird_ctx {
   // RAS
   int32_t* sd_row0 = nullptr;
   int32_t* sd_node = nullptr;
-  int64_t* l_row_ptr = nullptr;
-  int32_t* l_col = nullptr;
   int32_t* l_gblk = nullptr;
-  int64_t* l_diag = nullptr;
-  int64_t* upd_ptr = nullptr;
-  int64_t* upd = nullptr;
-  int32_t* fwd_order = nullptr;
+  int4* frec = nullptr;
+  int64_t* fpair = nullptr;
+  int32_t* upd = nullptr;
   int32_t* fwd_lev = nullptr;
   int32_t* sd_fwd_lev0 = nullptr;
-  int32_t* bwd_order = nullptr;
-  int32_t* bwd_lev = nullptr;
-  int32_t* sd_bwd_lev0 = nullptr;
   int32_t* own_ptr = nullptr;
   int32_t* owner = nullptr;
   int32_t* sd_sched = nullptr;

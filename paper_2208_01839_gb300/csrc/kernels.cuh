@@ -177,18 +177,12 @@ struct RasDev {
   const int32_t* sd_sched;  // CTA b of a per-subdomain kernel works on subdomain sd_sched[b]
   const int32_t* sd_row0;
   const int32_t* sd_node;
-  const int64_t* l_row_ptr;
-  const int32_t* l_col;
   const int32_t* l_gblk;
-  const int64_t* l_diag;
-  const int64_t* upd_ptr;
-  const int64_t* upd;
-  const int32_t* fwd_order;
+  const int4* frec;      // factorisation: row records in forward order (HostSetup::frec)
+  const int64_t* fpair;  // first update pair of each
+  const int2* upd;       // (destination | lower block << 16, source block)
   const int32_t* fwd_lev;
   const int32_t* sd_fwd_lev0;
-  const int32_t* bwd_order;
-  const int32_t* bwd_lev;
-  const int32_t* sd_bwd_lev0;
   const int32_t* own_ptr;
   double* fval;
   double* dinv;
@@ -214,8 +208,7 @@ constexpr int32_t SOLVE_WAIT_POLLS_DEFAULT = 1 << 20;
 void launch_ilu_factor(const RasDev& d, const double* val, const float* val32, int32_t* err, bool fp32,
                        cudaStream_t s);
 void launch_ilu_reorg(const RasDev& d, int64_t nfwd, int64_t nbwd, const int64_t* fsrc, const int32_t* fcol,
-                      const int32_t* frow, const int64_t* bsrc, const int32_t* bcol, const int32_t* brow, bool fp32,
-                      cudaStream_t s);
+                      const int32_t* frow, const int64_t* bsrc, const int32_t* bcol, bool fp32, cudaStream_t s);
 void launch_ilu_solve(const RasDev& d, const double* r, double* z, int32_t* err, cudaStream_t s);
 // r in FP32, rows padded to eight values (launch_pack32, launch_az_sub32)
 void launch_ilu_solve32(const RasDev& d, const float* r, float* z, int32_t* err, cudaStream_t s);

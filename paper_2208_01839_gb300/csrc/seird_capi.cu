@@ -322,18 +322,12 @@ RasDev ras_dev(seird_ctx* ctx) {
   d.sd_sched = ctx->sd_sched;
   d.sd_row0 = ctx->sd_row0;
   d.sd_node = ctx->sd_node;
-  d.l_row_ptr = ctx->l_row_ptr;
-  d.l_col = ctx->l_col;
   d.l_gblk = ctx->l_gblk;
-  d.l_diag = ctx->l_diag;
-  d.upd_ptr = ctx->upd_ptr;
-  d.upd = ctx->upd;
-  d.fwd_order = ctx->fwd_order;
+  d.frec = ctx->frec;
+  d.fpair = ctx->fpair;
+  d.upd = reinterpret_cast<const int2*>(ctx->upd);
   d.fwd_lev = ctx->fwd_lev;
   d.sd_fwd_lev0 = ctx->sd_fwd_lev0;
-  d.bwd_order = ctx->bwd_order;
-  d.bwd_lev = ctx->bwd_lev;
-  d.sd_bwd_lev0 = ctx->sd_bwd_lev0;
   d.own_ptr = ctx->own_ptr;
   d.fval = ctx->fval;
   d.dinv = ctx->dinv;
@@ -393,7 +387,7 @@ int pc_setup(seird_ctx* ctx) {
     const RasDev d = ras_dev(ctx);
     launch_ilu_factor(d, ctx->val, ctx->val32, ctx->err, mixed(ctx), ctx->stream);
     launch_ilu_reorg(d, (int64_t)ctx->hs.sp_fwd.src.size(), (int64_t)ctx->hs.sp_bwd.src.size(), ctx->pf.src,
-                     ctx->pf.col, ctx->pf.brow, ctx->pb.src, ctx->pb.col, ctx->pb.brow, mixed(ctx), ctx->stream);
+                     ctx->pf.col, ctx->pf.brow, ctx->pb.src, ctx->pb.col, mixed(ctx), ctx->stream);
   }
   CK(cudaGetLastError());
   if (ctx->opt.coarse) {
@@ -1543,18 +1537,12 @@ static int create_impl(seird_ctx* ctx, const seird_mesh* mesh, const seird_param
   // RAS
   TRY(upload(ctx, &ctx->sd_row0, hs.sd_row0));
   TRY(upload(ctx, &ctx->sd_node, hs.sd_node));
-  TRY(upload(ctx, &ctx->l_row_ptr, hs.l_row_ptr));
-  TRY(upload(ctx, &ctx->l_col, hs.l_col));
   TRY(upload(ctx, &ctx->l_gblk, hs.l_gblk));
-  TRY(upload(ctx, &ctx->l_diag, hs.l_diag));
-  TRY(upload(ctx, &ctx->upd_ptr, hs.upd_ptr));
+  TRY(upload(ctx, &ctx->frec, hs.frec));
+  TRY(upload(ctx, &ctx->fpair, hs.fpair));
   TRY(upload(ctx, &ctx->upd, hs.upd));
-  TRY(upload(ctx, &ctx->fwd_order, hs.fwd_order));
   TRY(upload(ctx, &ctx->fwd_lev, hs.fwd_lev));
   TRY(upload(ctx, &ctx->sd_fwd_lev0, hs.sd_fwd_lev0));
-  TRY(upload(ctx, &ctx->bwd_order, hs.bwd_order));
-  TRY(upload(ctx, &ctx->bwd_lev, hs.bwd_lev));
-  TRY(upload(ctx, &ctx->sd_bwd_lev0, hs.sd_bwd_lev0));
   TRY(upload(ctx, &ctx->own_ptr, hs.own_ptr));
   TRY(upload(ctx, &ctx->owner, hs.owner));
   TRY(upload(ctx, &ctx->sd_sched, hs.sd_sched));
@@ -1564,7 +1552,7 @@ static int create_impl(seird_ctx* ctx, const seird_mesh* mesh, const seird_param
     const HostSetup::SolvePlan& sp = dir == 0 ? hs.sp_fwd : hs.sp_bwd;
     seird_ctx::PlanPtrs& q = dir == 0 ? ctx->pf : ctx->pb;
     TRY(upload(ctx, &q.stage, sp.stage));
-    TRY(upload(ctx, &q.brow, sp.brow));
+    if (dir == 0) TRY(upload(ctx, &q.brow, sp.brow));
     TRY(upload(ctx, &q.sd_lev0, sp.sd_lev0));
     TRY(upload(ctx, &q.src, sp.src));
     TRY(upload(ctx, &q.col, sp.col));

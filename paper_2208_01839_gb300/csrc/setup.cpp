@@ -440,7 +440,7 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
     std::vector<int64_t> rowend;         // end of each local row's blocks
     std::vector<int32_t> l_col, l_gblk;  // local column and J block of each local block
     std::vector<int64_t> diag;           // diagonal block of each row
-    std::vector<int64_t> upd;            // ILU(0) update pairs (destination, source)
+    std::vector<int32_t> upd;            // update pairs (destination and lower block within the row, source)
     std::vector<int64_t> updend;         // pairs issued up to and including each block
     std::vector<int32_t> order[2], lb[2];
   };
@@ -506,8 +506,8 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
             for (int64_t b = rstart[k]; b < rstart[k + 1]; ++b) {
               const int32_t j = S.l_col[b];
               if (j > k && rowpos[j] >= 0) {
-                S.upd.push_back(rowpos[j]);
-                S.upd.push_back(b);
+                S.upd.push_back((int32_t)((rowpos[j] - rstart[i]) | (a - rstart[i]) << 16));
+                S.upd.push_back((int32_t)b);
               }
             }
           }
@@ -620,7 +620,10 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
       std::copy(S.l_col.begin(), S.l_col.end(), hs.l_col.begin() + b0);
       std::copy(S.l_gblk.begin(), S.l_gblk.end(), hs.l_gblk.begin() + b0);
       for (size_t a = 0; a < S.updend.size(); ++a) hs.upd_ptr[b0 + a + 1] = u0 + S.updend[a];
-      for (size_t k = 0; k < S.upd.size(); ++k) hs.upd[2 * u0 + k] = b0 + S.upd[k];
+      for (size_t k = 0; k < S.upd.size(); k += 2) {
+        hs.upd[2 * u0 + k] = S.upd[k];
+        hs.upd[2 * u0 + k + 1] = (int32_t)(b0 + S.upd[k + 1]);
+      }
       for (int dir = 0; dir < 2; ++dir) {
         std::vector<int32_t>& order = dir == 0 ? hs.fwd_order : hs.bwd_order;
         std::vector<int32_t>& levs = dir == 0 ? hs.fwd_lev : hs.bwd_lev;
@@ -747,6 +750,17 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
     hs.max_row_blocks = std::max<int64_t>({hs.max_row_blocks, hs.l_diag[R] - hs.l_row_ptr[R],
                                            hs.l_row_ptr[R + 1] - hs.l_diag[R]});
   parallel_for(P, setup_threads(P), [&](int32_t q, int) { place_stages(hs, q); });
+  // the factorisation's row records, in forward order
+  hs.frec.resize(hs.l_diag.size());
+  hs.fpair.resize(hs.l_diag.size());
+  parallel_for(P, setup_threads(P), [&](int32_t q, int) {
+    for (int64_t k = hs.sd_row0[q]; k < hs.sd_row0[q + 1]; ++k) {
+      const int64_t R = (int64_t)hs.sd_row0[q] + hs.fwd_order[k], a0 = hs.l_row_ptr[R], dg = hs.l_diag[R];
+      hs.frec[k] = make_int4((int32_t)R, (int32_t)a0, (int32_t)(hs.l_row_ptr[R + 1] - a0) | (int32_t)(dg - a0) << 16,
+                             (int32_t)(hs.upd_ptr[dg] - hs.upd_ptr[a0]));
+      hs.fpair[k] = hs.upd_ptr[a0];
+    }
+  });
 
   // ---- launch order of the subdomain CTAs ------------------------------------
   // Subdomains differ in size (2k-8k nodes at 4096 subdomains) and several waves of
@@ -975,6 +989,21 @@ int64_t check_setup(const HostSetup& hs, std::string& first) {
       fail(found == jcols.size(), "a block of R_p J R_p^T is missing from the factor pattern");
     }
     for (int32_t i = hs.own_ptr[q]; i < hs.own_ptr[q + 1]; ++i) fail(seen[i] == q, "owned node outside its subdomain");
+    // factorisation records and update pairs: block (i, j) takes (i, k) times (k, j), k < i, k < j
+    for (int32_t k = r0; k < r1 && !bad; ++k) {
+      const int4 fr = hs.frec[k];
+      const int64_t R = (int64_t)r0 + hs.fwd_order[k], a0 = hs.l_row_ptr[R];
+      const int32_t nb = fr.z & 0xffff, nlow = fr.z >> 16;
+      fail(fr.x == R && fr.y == a0 && nb == hs.l_row_ptr[R + 1] - a0 && nlow == hs.l_diag[R] - a0, "factor row record");
+      int32_t last = 0;
+      for (int32_t t = 0; t < fr.w && !bad; ++t) {
+        const int32_t x = hs.upd[2 * (hs.fpair[k] + t)], src = hs.upd[2 * (hs.fpair[k] + t) + 1];
+        const int32_t dst = x & 0xffff, j = x >> 16, m = hs.l_col[a0 + std::min(j, nb - 1)];
+        fail(j >= last && j < nlow && dst > j && dst < nb, "update pair outside its row");
+        fail(src > hs.l_diag[r0 + m] && src < hs.l_row_ptr[r0 + m + 1] && hs.l_col[src] == hs.l_col[a0 + dst], "update pair's source");
+        last = j;
+      }
+    }
   }
   // solve plans: each stage fits the shared-memory rings, every dependency of a row
   // lies in an earlier stage, and the records number the entries by sweep position

@@ -65,3 +65,38 @@ def test_every_form_matches_the_oracle(count, precision):
     for o in outs[1:]:
         assert np.array_equal(outs[0], o)
     assert np.linalg.norm(outs[0] - ref) <= (1e-4 if precision else 1e-10) * np.linalg.norm(ref)
+
+
+def _wheel_strip(spokes, cells):
+    """Triangle fan of `spokes` triangles around one node, on a strip of cells: the hub's row
+    of the factors has spokes + 1 blocks."""
+    t = np.linspace(0.0, 2.0 * np.pi, spokes, endpoint=False)
+    xy = [np.array([[0.0, 0.0]]), np.stack([np.cos(t), np.sin(t)], 1)]
+    tri = [[0, 1 + k, 1 + (k + 1) % spokes] for k in range(spokes)]
+    sxy, stri = I.structured_mesh(cells, 4, x0=3.0, x1=5.0)
+    xy.append(sxy)
+    off = 1 + spokes
+    return np.concatenate(xy), np.concatenate([np.array(tri), stri + off]).astype(np.int32)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("spokes", [5, 30, 31, 32, 33, 40, 100])
+def test_rows_longer_than_a_warp_holds(spokes, precision):
+    """A hub node numbered last has a lower row of `spokes` blocks: on either side of the 32
+    blocks that a warp keeps in shared memory, and far beyond."""
+    xy, tri = _wheel_strip(spokes, 40)
+    n = len(xy)
+    flip = (n - 1 - tri).astype(np.int32)  # the hub last
+    xy, tri = xy[::-1].copy(), flip
+    p = I.params_ontario(40.0)
+    U0 = np.random.default_rng(spokes).uniform(1.0, 2.0, (n, 5))
+    owner = np.zeros(n, dtype=np.int32)
+    rp, col, val = O.to_bsr(O.jacobian(xy, tri, p, 0.5, U0))
+    r = np.random.default_rng(1).standard_normal(5 * n)
+    ref = O.ras_apply(rp, col, val, owner, 0, r, coarse=False, ilu_fill=1)
+    with S.Solver(xy, tri, p, owner=owner, dt=0.5, overlap=0, ilu_fill=1, precision=precision) as sv:
+        sv.jacobian(U0)
+        sv.precond_setup()
+        got = sv.precond_apply(r.reshape(-1, 5)).ravel()
+    assert np.linalg.norm(got - ref) <= (1e-4 if precision else 1e-10) * np.linalg.norm(ref)
