@@ -84,7 +84,7 @@ void launch_norm2(int64_t len, const double* x, double* partial, int grid, doubl
 void launch_mdot(int64_t len, int nv, const double* V, int64_t ld, const double* w, double* partial, int grid,
                  double* out, cudaStream_t s, int tile = 0);
 void launch_update_mdot(int64_t len, int nv, const double* V, int64_t ld, const double* h, double* w,
-                        double* partial, int grid, double* out_add, cudaStream_t s, int tile = 0);
+                        double* partial, int grid, double* out, cudaStream_t s, int tile = 0);
 void launch_update_norm(int64_t len, int nv, const double* V, int64_t ld, const double* h, double* w,
                         double* partial, int grid, double* out, cudaStream_t s);
 void launch_scale(int64_t len, const double* x, const double* alpha_ptr, int invert, double* y, cudaStream_t s);

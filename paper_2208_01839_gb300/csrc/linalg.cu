@@ -3,6 +3,7 @@
 // FGMRES when the preconditioner varies).  FP64 accumulation throughout;
 // reductions are two-stage (per-CTA partials, then one CTA in fixed order), so
 // every result is bitwise reproducible run to run.
+#include <algorithm>
 #include <cmath>
 
 #include "kernels.cuh"
@@ -135,16 +136,16 @@ __global__ void __launch_bounds__(256) k_norm2_partial(int64_t len, const double
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
-// out[k] (+)= sum_cta partial[cta * stride + k], k < nv; fixed order
-__global__ void k_reduce_cols(int grid, int nv, int stride, const double* __restrict__ partial, double* out,
-                              int add) {
+// out[k] (+)= sum_cta partial[cta * stride + k], fixed order; CTA k sums column k (one CTA
+// for all columns took 15.7 us for 456 partials of 16 columns, which is 2.5 us this way)
+__global__ void __launch_bounds__(256) k_reduce_cols(int grid, int stride, const double* __restrict__ partial,
+                                                     double* out, int add) {
   __shared__ double sh[8];
-  for (int k = 0; k < nv; ++k) {
-    double s = 0.0;
-    for (int c = threadIdx.x; c < grid; c += blockDim.x) s += partial[(int64_t)c * stride + k];
-    s = block_sum<256>(s, sh);
-    if (threadIdx.x == 0) out[k] = add ? out[k] + s : s;
-  }
+  const int k = blockIdx.x;
+  double s = 0.0;
+  for (int c = threadIdx.x; c < grid; c += blockDim.x) s += partial[(int64_t)c * stride + k];
+  s = block_sum<256>(s, sh);
+  if (threadIdx.x == 0) out[k] = add ? out[k] + s : s;
 }
 
 constexpr int KPW = (NVMAX + 7) / 8;  // dot products per warp
@@ -230,13 +231,28 @@ __global__ void __launch_bounds__(256) k_cgs_db(int64_t len, int nv, const doubl
   }
 }
 
-// tile entries per CTA step: the caller's choice (128 or 256; 0 = by depth), 128 whenever
-// 256 would not fit twice in shared memory
-inline int cgs_tile(int nv, int want = 0) {
+inline size_t cgs_db_smem(int nv, int T) { return sizeof(double) * (NVMAX + 7 + T + 2 * (size_t)(nv + 1) * T); }
+
+// tile entries per CTA step: the caller's choice (128 or 256; 0 = by length and depth), 128
+// whenever 256 would not fit twice in shared memory, and 64 for vectors that would otherwise
+// leave SMs without a tile (5445 entries, 16 vectors: 13.5 us a pass with 22 CTAs of 256)
+inline int cgs_tile(int64_t len, int nv, int want = 0) {
+  if (want == 0 && len <= 152 * 128) return 64;
   if (nv > 27) return 128;
   return want == 128 ? 128 : 256;
 }
-inline size_t cgs_db_smem(int nv, int T) { return sizeof(double) * (NVMAX + 7 + T + 2 * (size_t)(nv + 1) * T); }
+// CTAs of a pass: no more than there are tiles (the rest would only add zeros to the sums)
+inline int cgs_grid(int64_t len, int T, int grid) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(grid, (len + T - 1) / T));
+}
+template <int MODE>
+void launch_cgs_db(int T, int64_t len, int nv, const double* V, int64_t ld, const double* h, double* w,
+                   double* partial, int grid, cudaStream_t s) {
+  const size_t sm = cgs_db_smem(nv, T);
+  if (T == 256) k_cgs_db<MODE, 256><<<grid, 256, sm, s>>>(len, nv, V, ld, h, w, partial);
+  else if (T == 128) k_cgs_db<MODE, 128><<<grid, 256, sm, s>>>(len, nv, V, ld, h, w, partial);
+  else k_cgs_db<MODE, 64><<<grid, 256, sm, s>>>(len, nv, V, ld, h, w, partial);
+}
 
 // second CGS pass update and ||w||^2 without staging: every thread needs only its
 // own entries of the basis vectors, so they go straight to registers
@@ -303,61 +319,82 @@ __global__ void k_multi_axpy(int64_t len, int nv, const double* __restrict__ Z, 
 // next iteration (cc.next) only while the outcome is 0 and the limit is not reached.
 __global__ void k_givens(int j, double* gm, const double* __restrict__ h1, const double* __restrict__ h2,
                          const double* __restrict__ hnext_sq, int ldh, double* out_res, CycleCtl cc) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int restart = ldh - 1;
+  // the warp brings the column, the rotations and the scalars on chip at once; the chain of
+  // rotations is one thread's, and the warp writes the column (one thread alone took 9 us at
+  // j = 16, nearly all of it waiting for its loads one after the other)
+  __shared__ double col[NVMAX + 1], rc[NVMAX], rs[NVMAX];
+  const int restart = ldh - 1, lane = threadIdx.x;
   double* H = gm;
   double* cs = H + (int64_t)ldh * restart;
   double* sn = cs + restart;
   double* g = sn + restart;
-  double col[NVMAX];
-  for (int k = 0; k <= j; ++k) col[k] = h1[k] + h2[k];  // CGS2: both passes' coefficients
+  for (int k = lane; k <= j; k += 32) {
+    col[k] = h1[k] + h2[k];  // CGS2: both passes' coefficients
+    if (k < j) {
+      rc[k] = cs[k];
+      rs[k] = sn[k];
+    }
+  }
   const double hn = sqrt(fmax(*hnext_sq, 0.0));
-  col[j + 1] = hn;
-  for (int k = 0; k < j; ++k) {
-    const double a = col[k], b = col[k + 1];
-    col[k] = cs[k] * a + sn[k] * b;
-    col[k + 1] = -sn[k] * a + cs[k] * b;
-  }
-  const double a = col[j], b = col[j + 1];
-  const double rr = hypot(a, b);
-  double c = 1.0, s = 0.0;
-  if (rr != 0.0) {
-    c = a / rr;
-    s = b / rr;
-  }
-  cs[j] = c;
-  sn[j] = s;
-  col[j] = rr;
-  col[j + 1] = 0.0;
-  for (int k = 0; k <= j + 1; ++k) H[k + (int64_t)ldh * j] = col[k];
   const double gj = g[j];
-  g[j] = c * gj;
-  g[j + 1] = -s * gj;
-  out_res[0] = fabs(g[j + 1]);
-  out_res[1] = hn;
-  if (cc.ctl) {
-    const double res = fabs(g[j + 1]);
-    int outcome = 0;
-    if (!(res <= cc.tol[1]) || !isfinite(res)) outcome = 2;
-    else if (res <= cc.tol[0] || hn == 0.0) outcome = 1;
-    cc.ctl[0] = j + 1;
-    cc.ctl[2] = outcome;
-    if (cc.has_next) cudaGraphSetConditional(cc.next, (outcome == 0 && j + 1 < cc.ctl[1]) ? 1u : 0u);
+  __syncwarp();
+  if (lane == 0) {
+    double a = col[0];
+    for (int k = 0; k < j; ++k) {
+      const double b = col[k + 1];
+      col[k] = rc[k] * a + rs[k] * b;
+      a = -rs[k] * a + rc[k] * b;
+    }
+    const double b = hn;
+    const double rr = hypot(a, b);
+    double c = 1.0, s = 0.0;
+    if (rr != 0.0) {
+      c = a / rr;
+      s = b / rr;
+    }
+    cs[j] = c;
+    sn[j] = s;
+    col[j] = rr;
+    col[j + 1] = 0.0;
+    g[j] = c * gj;
+    const double gn = -s * gj;
+    g[j + 1] = gn;
+    const double res = fabs(gn);
+    out_res[0] = res;
+    out_res[1] = hn;
+    if (cc.ctl) {
+      int outcome = 0;
+      if (!(res <= cc.tol[1]) || !isfinite(res)) outcome = 2;
+      else if (res <= cc.tol[0] || hn == 0.0) outcome = 1;
+      cc.ctl[0] = j + 1;
+      cc.ctl[2] = outcome;
+      if (cc.has_next) cudaGraphSetConditional(cc.next, (outcome == 0 && j + 1 < cc.ctl[1]) ? 1u : 0u);
+    }
   }
+  __syncwarp();
+  for (int k = lane; k <= j + 1; k += 32) H[k + (int64_t)ldh * j] = col[k];
 }
 
-// y = H(0:k,0:k)^{-1} g(0:k) by back substitution (one thread)
-__global__ void k_hsolve(int k, double* gm, int ldh) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// y = H(0:k,0:k)^{-1} g(0:k) by back substitution: the CTA brings the triangle on chip, one
+// thread solves
+__global__ void __launch_bounds__(256) k_hsolve(int k, double* gm, int ldh) {
+  extern __shared__ double hs[];  // [k][k] column-major, then g
   const int restart = ldh - 1;
-  double* H = gm;
-  double* g = H + (int64_t)ldh * restart + 2 * restart;
+  const double* H = gm;
+  double* g = gm + (int64_t)ldh * restart + 2 * restart;
   double* y = g + ldh;
+  for (int q = threadIdx.x; q < k * k; q += blockDim.x) hs[q] = H[q % k + (int64_t)ldh * (q / k)];
+  double* v = hs + k * k;
+  for (int q = threadIdx.x; q < k; q += blockDim.x) v[q] = g[q];
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   for (int i = k - 1; i >= 0; --i) {
-    double v = g[i];
-    for (int c = i + 1; c < k; ++c) v -= H[i + (int64_t)ldh * c] * y[c];
-    const double d = H[i + (int64_t)ldh * i];
-    y[i] = d != 0.0 ? v / d : 0.0;
+    double t = v[i];
+    for (int c = i + 1; c < k; ++c) t -= hs[i + k * c] * v[c];
+    const double d = hs[i + k * i];
+    t = d != 0.0 ? t / d : 0.0;
+    v[i] = t;
+    y[i] = t;
   }
 }
 
@@ -434,41 +471,37 @@ void launch_f32_to_f64(int64_t n, const float* src, double* dst, cudaStream_t s)
 }
 
 void launch_norm2(int64_t len, const double* x, double* partial, int grid, double* out, cudaStream_t s) {
-  k_norm2_partial<<<grid, 256, 0, s>>>(len, x, partial);
-  k_reduce_cols<<<1, 256, 0, s>>>(grid, 1, 1, partial, out, 0);
+  const int g = cgs_grid(len, 256, grid);
+  k_norm2_partial<<<g, 256, 0, s>>>(len, x, partial);
+  k_reduce_cols<<<1, 256, 0, s>>>(g, 1, partial, out, 0);
   count_launch();
   count_launch();
 }
 
 void launch_mdot(int64_t len, int nv, const double* V, int64_t ld, const double* w, double* partial, int grid,
                  double* out, cudaStream_t s, int tile) {
-  if (cgs_tile(nv, tile) == 256)
-    k_cgs_db<0, 256><<<grid, 256, cgs_db_smem(nv, 256), s>>>(len, nv, V, ld, nullptr, const_cast<double*>(w),
-                                                            partial);
-  else
-    k_cgs_db<0, 128><<<grid, 256, cgs_db_smem(nv, 128), s>>>(len, nv, V, ld, nullptr, const_cast<double*>(w),
-                                                            partial);
-  k_reduce_cols<<<1, 256, 0, s>>>(grid, nv, NVMAX, partial, out, 0);
+  const int T = cgs_tile(len, nv, tile), g = cgs_grid(len, T, grid);
+  launch_cgs_db<0>(T, len, nv, V, ld, nullptr, const_cast<double*>(w), partial, g, s);
+  k_reduce_cols<<<nv, 256, 0, s>>>(g, NVMAX, partial, out, 0);
   count_launch();
   count_launch();
 }
 
-// first CGS pass update fused with the second pass's dot products; the dots
-// are added to out_add (which holds the first-pass coefficients h)
+// first CGS pass update fused with the second pass's dot products (to out)
 void launch_update_mdot(int64_t len, int nv, const double* V, int64_t ld, const double* h, double* w,
-                        double* partial, int grid, double* out_add, cudaStream_t s, int tile) {
-  if (cgs_tile(nv, tile) == 256)
-    k_cgs_db<1, 256><<<grid, 256, cgs_db_smem(nv, 256), s>>>(len, nv, V, ld, h, w, partial);
-  else
-    k_cgs_db<1, 128><<<grid, 256, cgs_db_smem(nv, 128), s>>>(len, nv, V, ld, h, w, partial);
+                        double* partial, int grid, double* out, cudaStream_t s, int tile) {
+  const int T = cgs_tile(len, nv, tile), g = cgs_grid(len, T, grid);
+  launch_cgs_db<1>(T, len, nv, V, ld, h, w, partial, g, s);
+  k_reduce_cols<<<nv, 256, 0, s>>>(g, NVMAX, partial, out, 0);
   count_launch();
-  (void)out_add;
+  count_launch();
 }
 
 void launch_update_norm(int64_t len, int nv, const double* V, int64_t ld, const double* h, double* w,
                         double* partial, int grid, double* out, cudaStream_t s) {
-  k_cgs_update_norm<<<grid, 256, 0, s>>>(len, nv, V, ld, h, w, partial);
-  k_reduce_cols<<<1, 256, 0, s>>>(grid, 1, NVMAX, partial, out, 0);
+  const int g = cgs_grid(len, 256, grid);
+  k_cgs_update_norm<<<g, 256, 0, s>>>(len, nv, V, ld, h, w, partial);
+  k_reduce_cols<<<1, 256, 0, s>>>(g, NVMAX, partial, out, 0);
   count_launch();
   count_launch();
 }
@@ -479,10 +512,12 @@ void cgs_init() {
   cudaFuncSetAttribute(k_cgs_db<1, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_cgs_db<0, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   cudaFuncSetAttribute(k_cgs_db<1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  cudaFuncSetAttribute(k_cgs_db<0, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  cudaFuncSetAttribute(k_cgs_db<1, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
 }
 
 void launch_reduce_cols(int grid, int nv, const double* partial, double* out, int add, cudaStream_t s) {
-  k_reduce_cols<<<1, 256, 0, s>>>(grid, nv, NVMAX, partial, out, add);
+  k_reduce_cols<<<nv, 256, 0, s>>>(grid, NVMAX, partial, out, add);
   count_launch();
 }
 
@@ -509,7 +544,7 @@ void launch_givens(int j, double* gm, const double* h1, const double* h2, const 
 }
 
 void launch_hsolve(int k, double* gm, int ldh, cudaStream_t s) {
-  k_hsolve<<<1, 32, 0, s>>>(k, gm, ldh);
+  k_hsolve<<<1, 256, sizeof(double) * (size_t)k * (k + 1), s>>>(k, gm, ldh);
   count_launch();
 }
 

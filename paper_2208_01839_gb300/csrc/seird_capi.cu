@@ -728,9 +728,7 @@ static int arnoldi_iteration(seird_ctx* ctx, int j, const CycleCtl& cc) {
   if (ctx->opt.gmres_one_pass == 1) {
     launch_update_norm(len, j + 1, ctx->V, len, h1, ctx->w, ctx->partial, ctx->red_grid, ctx->scal + 5, s);
   } else {
-    launch_update_mdot(len, j + 1, ctx->V, len, h1, ctx->w, ctx->partial, ctx->red_grid, nullptr, s,
-                       ctx->cgs_tile);
-    launch_reduce_cols(ctx->red_grid, j + 1, ctx->partial, h2, 0, s);
+    launch_update_mdot(len, j + 1, ctx->V, len, h1, ctx->w, ctx->partial, ctx->red_grid, h2, s, ctx->cgs_tile);
     launch_update_norm(len, j + 1, ctx->V, len, h2, ctx->w, ctx->partial, ctx->red_grid, ctx->scal + 5, s);
   }
   launch_givens(j, ctx->gm, h1, h2, ctx->scal + 5, ldh, ctx->scal + 2, s, cc);
@@ -1515,7 +1513,8 @@ static int create_impl(seird_ctx* ctx, const seird_mesh* mesh, const seird_param
   } else {
     TRY(dalloc(ctx, &ctx->Z, (size_t)R * len));
   }
-  const int64_t npart = std::max<int64_t>((int64_t)ctx->sms * 6 * NV_STRIDE, (n + 255) / 256);  // up to 6 CTAs/SM
+  // a row for every CTA that seird_set_launch_shapes may ask for (64 per SM)
+  const int64_t npart = std::max<int64_t>((int64_t)ctx->sms * 64 * NV_STRIDE, (n + 255) / 256);
   if (o.autotune) TRY(dalloc(ctx, &ctx->tune_buf, len));
   TRY(dalloc(ctx, &ctx->partial, npart));
   TRY(dalloc(ctx, &ctx->hcol, 2 * NV_STRIDE));
