@@ -78,6 +78,10 @@ void launch_jacobian(int64_t nnzb, int64_t m, const int32_t* tri, const double* 
 template <class VT>
 void launch_spmv(int64_t nrow, const int32_t* rp, const int32_t* col, const VT* val, const double* x, double* y,
                  cudaStream_t s, int tb = 256, const double* b = nullptr);
+// y = A x for a caller's own matrix, whose rows may differ in length
+template <class VT>
+void launch_spmv_uneven(int64_t nrow, const int32_t* rp, const int32_t* col, const VT* val, const double* x, double* y,
+                        cudaStream_t s);
 
 // vectors (length len, grid-stride)
 void launch_norm2(int64_t len, const double* x, double* partial, int grid, double* out, cudaStream_t s);

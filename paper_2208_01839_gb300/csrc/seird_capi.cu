@@ -1959,7 +1959,7 @@ int seird_bsr_spmv(int64_t n_rows, const int32_t* row_ptr, const int32_t* col, c
   if (n_rows < 0) return SEIRD_EINVAL;
   if (n_rows == 0) return SEIRD_OK;
   if (!row_ptr || !col || !val || !x || !y) return SEIRD_EINVAL;
-  launch_spmv<double>(n_rows, row_ptr, col, val, x, y, (cudaStream_t)stream);
+  launch_spmv_uneven<double>(n_rows, row_ptr, col, val, x, y, (cudaStream_t)stream);
   return cudaGetLastError() == cudaSuccess ? SEIRD_OK : SEIRD_ECUDA;
 }
 
@@ -1968,7 +1968,7 @@ int seird_bsr_spmv_f32val(int64_t n_rows, const int32_t* row_ptr, const int32_t*
   if (n_rows < 0) return SEIRD_EINVAL;
   if (n_rows == 0) return SEIRD_OK;
   if (!row_ptr || !col || !val || !x || !y) return SEIRD_EINVAL;
-  launch_spmv<float>(n_rows, row_ptr, col, val, x, y, (cudaStream_t)stream);
+  launch_spmv_uneven<float>(n_rows, row_ptr, col, val, x, y, (cudaStream_t)stream);
   return cudaGetLastError() == cudaSuccess ? SEIRD_OK : SEIRD_ECUDA;
 }
 
