@@ -14,15 +14,6 @@ namespace {
 
 constexpr int NVMAX = 65;  // restart <= 64 -> at most 65 basis vectors
 
-// (double)f on the integer pipe: GB300 converts at its FP64 rate, so a conversion costs as much
-// as the FMA it feeds.  The exponent is rebiased (127 -> 1023) and the 23 fraction bits become
-// the leading ones of 52; subnormals, infinities and NaNs take the conversion instruction.
-__device__ __forceinline__ double widen(float f) {
-  const uint32_t b = __float_as_uint(f), m = b & 0x7fffffffu;
-  if (m - 0x00800000u >= 0x7f000000u && m != 0) return (double)f;
-  const uint32_t hi = m ? (m >> 3) + 0x38000000u : 0u;
-  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
-}
 __device__ __forceinline__ double ld_val(const double* p) { return __ldg(p); }
 __device__ __forceinline__ double ld_val(const float* p) { return widen(__ldg(p)); }
 

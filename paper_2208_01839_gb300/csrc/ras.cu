@@ -775,8 +775,18 @@ __global__ void k_coarse_chunks(int32_t nchunk, const int32_t* __restrict__ cptr
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (gw >= nchunk || lane >= 25) return;
+  // eight blocks in flight (the sums stay in block order): 2.0M nodes 0.87 ms with one
   double s = 0.0;
-  for (int32_t b = cptr[gw]; b < cptr[gw + 1]; ++b) s += (double)val[25 * (int64_t)blk[b] + lane];
+  const int32_t e = cptr[gw + 1];
+  int32_t b = cptr[gw];
+  for (; b + 8 <= e; b += 8) {
+    TV v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = val[25 * (int64_t)blk[b + u] + lane];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += widen(v[u]);
+  }
+  for (; b < e; ++b) s += widen(val[25 * (int64_t)blk[b] + lane]);
   cpart[25 * gw + lane] = s;
 }
 
@@ -795,41 +805,43 @@ __device__ __forceinline__ double* bblk(double* band, int bw, int ib, int jb) {
   return band + 25 * ((int64_t)ib * (2 * bw + 1) + (jb - ib + bw));
 }
 
-// block step kb: invert the pivot block, form the L column below it
-__global__ void k_band_pivot(int P, int bw, int kb, double* band, double* cdinv, int32_t* err) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (warp == 0) warp_inv5<double>(bblk(band, bw, kb, kb), cdinv + 25 * (int64_t)kb, lane, err);
-  __syncthreads();
-  const double* Dk = cdinv + 25 * (int64_t)kb;
-  const int rr = lane / 5, cc = lane % 5;
-  const int last = min(P - 1, kb + bw);
-  for (int ib = kb + 1 + warp; ib <= last; ib += nw) {
-    double* A = bblk(band, bw, ib, kb);
-    double v = 0.0;
-    if (lane < 25) {
-#pragma unroll
-      for (int mm = 0; mm < 5; ++mm) v = fma(A[5 * rr + mm], Dk[5 * mm + cc], v);
-    }
+// Block step kb of the banded LU, one CTA per row i in (kb, kb + bw] (one in all at the end):
+// every CTA inverts the pivot block for itself (the step's latency either way), forms
+// L_i,kb and updates its row, A_ij -= L_i,kb A_kb,j for j in (kb, kb + bw]; no CTA writes
+// what another reads, so a step is one launch.  512 units, half-bandwidth 28: 9.2 us a step
+// with a launch for the pivot column and one for the update, 4.8 us now.
+__global__ void __launch_bounds__(256) k_band_step(int P, int bw, int kb, double* band, double* cdinv, int32_t* err) {
+  __shared__ double Dk[25], L[25];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nb = min(bw, P - 1 - kb), ib = kb + 1 + blockIdx.x;
+  if (warp == 0) {
+    const double a = lane < 25 && nb > 0 ? bblk(band, bw, ib, kb)[lane] : 0.0;
+    warp_inv5<double>(bblk(band, bw, kb, kb), Dk, lane, err);
     __syncwarp();
-    if (lane < 25) A[lane] = v;
-  }
-}
-
-// block step kb: trailing update A_ij -= L_ik A_kj for i, j in (kb, kb+bw]
-__global__ void k_band_update(int P, int bw, int kb, double* band) {
-  const int nb = min(bw, P - 1 - kb);
-  const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t pair = g / 25;
-  if (pair >= (int64_t)nb * nb) return;
-  const int e = (int)(g - 25 * pair);
-  const int ib = kb + 1 + (int)(pair / nb), jb = kb + 1 + (int)(pair % nb);
-  const int rr = e / 5, cc = e % 5;
-  const double* L = bblk(band, bw, ib, kb);
-  const double* Ak = bblk(band, bw, kb, jb);
-  double v = 0.0;
+    if (blockIdx.x == 0 && lane < 25) cdinv[25 * (int64_t)kb + lane] = Dk[lane];
+    if (nb > 0) {
+      const int rr = lane / 5, cc = lane - 5 * rr;
+      double v = 0.0;
 #pragma unroll
-  for (int mm = 0; mm < 5; ++mm) v = fma(L[5 * rr + mm], Ak[5 * mm + cc], v);
-  bblk(band, bw, ib, jb)[e] -= v;
+      for (int mm = 0; mm < 5; ++mm) {
+        const double am = __shfl_sync(FULL, a, (5 * rr + mm) & 31);
+        if (lane < 25) v = fma(am, Dk[5 * mm + cc], v);
+      }
+      if (lane < 25) {
+        L[lane] = v;
+        bblk(band, bw, ib, kb)[lane] = v;
+      }
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < 25 * nb; t += blockDim.x) {
+    const int jb = kb + 1 + t / 25, e = t % 25, rr = e / 5, cc = e - 5 * rr;
+    const double* Ak = bblk(band, bw, kb, jb);
+    double v = 0.0;
+#pragma unroll
+    for (int mm = 0; mm < 5; ++mm) v = fma(L[5 * rr + mm], Ak[5 * mm + cc], v);
+    bblk(band, bw, ib, jb)[e] -= v;
+  }
 }
 
 // y <- A_c^{-1} y with the banded block LU factors (one CTA, y in shared memory).
@@ -886,7 +898,10 @@ __global__ void k_band_solve(int P, int bw, const double* __restrict__ band, con
 // Explicit inverse, one CTA per block column b of the identity: L U X = E_b for
 // its five columns at once (ys[row][c] in shared memory), so a step over one
 // block row of the band is 25 independent dot products per band block.  X goes
-// to rows 5b..5b+4 of AinvT (row j of AinvT = column j of A_c^{-1}).
+// to rows 5b..5b+4 of AinvT (row j of AinvT = column j of A_c^{-1}).  Bound by the FP64 pipe
+// (five FMAs a product sum) and by the latency of a step's band blocks, which are
+// therefore loaded a step ahead, INV_ITEMS sums a thread (512 units: 5.36 ms without).
+constexpr int INV_ITEMS = 3;
 __global__ void __launch_bounds__(256) k_band_inv(int P, int bw, const double* __restrict__ band,
                                                   const double* __restrict__ cdinv, double* __restrict__ ainvT) {
   extern __shared__ double ys[];
@@ -894,39 +909,64 @@ __global__ void __launch_bounds__(256) k_band_inv(int P, int bw, const double* _
   const int b = blockIdx.x;
   double* bandm = const_cast<double*>(band);
   for (int k = tid; k < 25 * P; k += bd) ys[k] = (k / 5 == 5 * b + k % 5) ? 1.0 : 0.0;
+  // item t of step kb: row r of the band block t / 25 rows below (above) kb, column cc
+  auto rowp = [&](int kb, int t, bool fwd) {
+    return bblk(bandm, bw, fwd ? kb + 1 + t / 25 : kb - 1 - t / 25, kb) + 5 * ((t / 5) % 5);
+  };
+  double A[INV_ITEMS][5];
+  auto fetch = [&](int kb, bool fwd) {
+    const int n = 25 * (fwd ? min(bw, P - 1 - kb) : min(bw, kb));
+#pragma unroll
+    for (int u = 0; u < INV_ITEMS; ++u) {
+      const int t = tid + 256 * u;
+      if (t < n) {
+        const double* p = rowp(kb, t, fwd);
+#pragma unroll
+        for (int mm = 0; mm < 5; ++mm) A[u][mm] = __ldg(p + mm);
+      }
+    }
+  };
+  auto item = [&](int kb, int t, bool fwd, const double* a) {
+    const int ib = fwd ? kb + 1 + t / 25 : kb - 1 - t / 25, r = (t / 5) % 5, cc = t % 5;
+    double v = ys[5 * (5 * ib + r) + cc];
+#pragma unroll
+    for (int mm = 0; mm < 5; ++mm) v = fma(-a[mm], ys[5 * (5 * kb + mm) + cc], v);
+    ys[5 * (5 * ib + r) + cc] = v;
+  };
+  auto step = [&](int kb, bool fwd, int next) {
+    const int n = 25 * (fwd ? min(bw, P - 1 - kb) : min(bw, kb));
+#pragma unroll
+    for (int u = 0; u < INV_ITEMS; ++u)
+      if (tid + 256 * u < n) item(kb, tid + 256 * u, fwd, A[u]);
+    for (int t = tid + 256 * INV_ITEMS; t < n; t += 256) item(kb, t, fwd, rowp(kb, t, fwd));
+    if (next >= 0 && next < P) fetch(next, fwd);
+    __syncthreads();
+  };
+  fetch(b, true);
   __syncthreads();
-  for (int kb = b; kb < P; ++kb) {  // E_b is zero above block row b
-    const int nb = min(bw, P - 1 - kb);
-    for (int t = tid; t < 25 * nb; t += bd) {
-      const int ib = kb + 1 + t / 25, r = (t / 5) % 5, cc = t % 5;
-      const double* L = bblk(bandm, bw, ib, kb) + 5 * r;
-      double v = 0.0;
-#pragma unroll
-      for (int mm = 0; mm < 5; ++mm) v = fma(L[mm], ys[5 * (5 * kb + mm) + cc], v);
-      ys[5 * (5 * ib + r) + cc] -= v;
-    }
-    __syncthreads();
-  }
-  for (int kb = P - 1; kb >= 0; --kb) {
-    double tmp = 0.0;
+  for (int kb = b; kb < P; ++kb) step(kb, true, kb + 1);  // E_b is zero above block row b
+  fetch(P - 1, false);
+  double D[5];
+  auto pivot = [&](int kb) {
     if (tid < 25) {
-      const double* Dk = cdinv + 25 * (int64_t)kb + 5 * (tid / 5);
 #pragma unroll
-      for (int mm = 0; mm < 5; ++mm) tmp = fma(Dk[mm], ys[5 * (5 * kb + mm) + tid % 5], tmp);
+      for (int mm = 0; mm < 5; ++mm) D[mm] = __ldg(cdinv + 25 * (int64_t)kb + 5 * (tid / 5) + mm);
     }
-    __syncthreads();
-    if (tid < 25) ys[5 * (5 * kb + tid / 5) + tid % 5] = tmp;
-    __syncthreads();
-    const int nb = min(bw, kb);
-    for (int t = tid; t < 25 * nb; t += bd) {
-      const int ib = kb - 1 - t / 25, r = (t / 5) % 5, cc = t % 5;
-      const double* Ub = bblk(bandm, bw, ib, kb) + 5 * r;
-      double v = 0.0;
+  };
+  pivot(P - 1);
+  for (int kb = P - 1; kb >= 0; --kb) {
+    if (tid < 32) {  // one warp: its lanes read the five rows before they write them
+      double tmp = 0.0;
+      if (tid < 25) {
 #pragma unroll
-      for (int mm = 0; mm < 5; ++mm) v = fma(Ub[mm], ys[5 * (5 * kb + mm) + cc], v);
-      ys[5 * (5 * ib + r) + cc] -= v;
+        for (int mm = 0; mm < 5; ++mm) tmp = fma(D[mm], ys[5 * (5 * kb + mm) + tid % 5], tmp);
+      }
+      __syncwarp();
+      if (tid < 25) ys[5 * (5 * kb + tid / 5) + tid % 5] = tmp;
     }
+    if (kb > 0) pivot(kb - 1);
     __syncthreads();
+    step(kb, false, kb - 1);
   }
   const int64_t nc = 5 * (int64_t)P;
   for (int k = tid; k < 25 * P; k += bd) ainvT[(5 * b + k % 5) * nc + k / 5] = ys[k];
@@ -1120,14 +1160,8 @@ void launch_coarse_assemble(const CoarseDev& c, const double* val, const float* 
 
 void launch_coarse_factor(const CoarseDev& c, int32_t* err, cudaStream_t s) {
   for (int kb = 0; kb < c.P; ++kb) {
-    k_band_pivot<<<1, 256, 0, s>>>(c.P, c.band, kb, c.cband, c.cdinv, err);
+    k_band_step<<<std::max(1, std::min(c.band, c.P - 1 - kb)), 256, 0, s>>>(c.P, c.band, kb, c.cband, c.cdinv, err);
     count_launch();
-    const int nb = std::min(c.band, c.P - 1 - kb);
-    if (nb > 0) {
-      const int64_t th = 25 * (int64_t)nb * nb;
-      k_band_update<<<(int)((th + 255) / 256), 256, 0, s>>>(c.P, c.band, kb, c.cband);
-      count_launch();
-    }
   }
   if (c.ainvT) {  // explicit inverse through the banded factors
     if (25 * (size_t)c.P * sizeof(double) <= 227 * 1024) {  // a block column of five unit vectors per CTA
@@ -1196,7 +1230,7 @@ __global__ void k_az_build(int64_t nseg, const int32_t* __restrict__ az_blk, con
   const int64_t s = g / 25;
   const int e = (int)(g - 25 * s);
   double acc = 0.0;
-  for (int32_t b = az_blk[s]; b < az_blk[s + 1]; ++b) acc += (double)val[25 * (int64_t)b + e];
+  for (int32_t b = az_blk[s]; b < az_blk[s + 1]; ++b) acc += widen(val[25 * (int64_t)b + e]);
   azval[g] = (TA)acc;
 }
 
