@@ -209,8 +209,8 @@ struct seird_ctx {
   double* nodebuf = nullptr;  // [n][8] node terms of the residual
   double* scal = nullptr;   // scalar outputs (norms)
   double* h_scal = nullptr; // pinned host mirror
-  int32_t* err = nullptr;   // device error flags
-  int32_t* h_err = nullptr; // pinned
+  int32_t* err = nullptr;   // device error flags, in the last of the scalar outputs
+  int32_t* h_err = nullptr; // their host mirror, likewise
   int* dflag = nullptr;      // device flag of seird_set_state's comparison with the held state
   int* h_flag = nullptr;     // pinned
   int red_grid = 0;

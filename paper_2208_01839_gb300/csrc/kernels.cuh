@@ -129,7 +129,9 @@ void launch_reduce_cols(int grid, int nv, const double* partial, double* out, in
 void cgs_init();
 constexpr int NV_STRIDE = 65;  // row stride of the CGS partial-sum buffer
 void launch_hsolve(int k, double* gm, int ldh, cudaStream_t s);
-void launch_gather5(int64_t n, const int32_t* idx, const double* src, double* dst, cudaStream_t s);
+// dst[k] = src[idx[k]] (rows of five), and the same for a second pair when src2 != NULL
+void launch_gather5(int64_t n, const int32_t* idx, const double* src, double* dst, cudaStream_t s,
+                    const double* src2 = nullptr, double* dst2 = nullptr);
 void launch_scatter5(int64_t n, const int32_t* idx, const double* src, double* dst, cudaStream_t s);
 
 // discrete adjoint

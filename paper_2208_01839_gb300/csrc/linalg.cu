@@ -430,10 +430,12 @@ __global__ void __launch_bounds__(256) k_hsolve(int k, double* gm, int ldh) {
 }
 
 __global__ void k_gather5(int64_t n, const int32_t* __restrict__ idx, const double* __restrict__ src,
-                          double* __restrict__ dst) {
+                          double* __restrict__ dst, const double* __restrict__ src2, double* __restrict__ dst2) {
   for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < 5 * n; g += (int64_t)gridDim.x * blockDim.x) {
     const int64_t k = g / 5;
-    dst[g] = src[5 * (int64_t)idx[k] + (g - 5 * k)];
+    const int64_t f = 5 * (int64_t)idx[k] + (g - 5 * k);
+    dst[g] = src[f];
+    if (src2) dst2[g] = src2[f];
   }
 }
 
@@ -593,8 +595,9 @@ void launch_hsolve(int k, double* gm, int ldh, cudaStream_t s) {
   count_launch();
 }
 
-void launch_gather5(int64_t n, const int32_t* idx, const double* src, double* dst, cudaStream_t s) {
-  k_gather5<<<grid_for(5 * n), 256, 0, s>>>(n, idx, src, dst);
+void launch_gather5(int64_t n, const int32_t* idx, const double* src, double* dst, cudaStream_t s,
+                    const double* src2, double* dst2) {
+  k_gather5<<<grid_for(5 * n), 256, 0, s>>>(n, idx, src, dst, src2, dst2);
   count_launch();
 }
 

@@ -154,8 +154,15 @@ int64_t vlen(const seird_ctx* ctx) { return 5 * ctx->hs.n; }
 
 bool mixed(const seird_ctx* ctx) { return ctx->opt.precision == 1; }
 
-int check_flags(seird_ctx* ctx, const char* where) {
-  CK(cudaMemcpyAsync(ctx->h_err, ctx->err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+// the device error word is the last of the scalar outputs, so that one copy brings both:
+// scalars from `first` on and the error word.  A copy costs the host as much as a launch, and
+// a small call is its launches and copies: a residual on 1089 nodes took 68.3 us with two
+// copies and a gather for each state, 61.6 us with one of each
+constexpr int SCAL_COUNT = 16, SCAL_ERR = SCAL_COUNT - 1;
+
+int check_flags(seird_ctx* ctx, const char* where, int first = SCAL_ERR) {
+  CK(cudaMemcpyAsync(ctx->h_scal + first, ctx->scal + first, sizeof(double) * (SCAL_COUNT - first),
+                     cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   const int32_t f = *ctx->h_err;
   if (!f) return SEIRD_OK;
@@ -292,8 +299,7 @@ int residual(seird_ctx* ctx, const double* U, const double* Un, double* F, doubl
                     ctx->scal, ctx->err, ctx->stream);
   }
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(ctx->h_scal, ctx->scal, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-  TRY(check_flags(ctx, "residual"));
+  TRY(check_flags(ctx, "residual", 0));
   const double v = ctx->h_scal[0];
   if (!std::isfinite(v)) return fail(ctx, SEIRD_ENONFINITE, "residual: non-finite norm");
   *fn = std::sqrt(v);
@@ -590,14 +596,7 @@ int read_scalars(seird_ctx* ctx, int first, int count) {
 
 // read_scalars plus the device error word in the same synchronisation: a set flag
 // (a subdomain solve that timed out, a singular pivot) ends the caller's loop at once
-int read_scalars_checked(seird_ctx* ctx, int first, int count, const char* where) {
-  CK(cudaMemcpyAsync(ctx->h_scal + first, ctx->scal + first, sizeof(double) * count, cudaMemcpyDeviceToHost,
-                     ctx->stream));
-  CK(cudaMemcpyAsync(ctx->h_err, ctx->err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
-  if (*ctx->h_err) return check_flags(ctx, where);
-  return SEIRD_OK;
-}
+int read_scalars_checked(seird_ctx* ctx, int first, const char* where) { return check_flags(ctx, where, first); }
 
 int norm2(seird_ctx* ctx, const double* x, double* out) {
   launch_norm2(vlen(ctx), x, ctx->partial, ctx->red_grid, ctx->scal + 4, ctx->stream);
@@ -868,7 +867,7 @@ int gmres(seird_ctx* ctx, const double* b, double* x, double rtol, int* its_out,
       CK(cudaMemcpyAsync(ctx->cyc_ctl, hin, 4 * sizeof(int), cudaMemcpyHostToDevice, s));
       CK(cudaGraphLaunch(ctx->cycle_exec, s));
       CK(cudaMemcpyAsync(hout, ctx->cyc_ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
-      TRY(read_scalars_checked(ctx, 2, 2, "gmres"));
+      TRY(read_scalars_checked(ctx, 2, "gmres"));
       k = hout[0];
       its += k;
       if (k < 1 || k > m) return fail(ctx, SEIRD_ECUDA, "gmres: captured cycle reported no iterations");
@@ -882,7 +881,7 @@ int gmres(seird_ctx* ctx, const double* b, double* x, double rtol, int* its_out,
     } else {
       for (int j = 0; j < m; ++j) {
         TRY(arnoldi_iteration(ctx, j, CycleCtl()));
-        TRY(read_scalars_checked(ctx, 2, 2, "gmres"));
+        TRY(read_scalars_checked(ctx, 2, "gmres"));
         ++its;
         k = j + 1;
         const double res = ctx->h_scal[2], hn = ctx->h_scal[3];
@@ -1431,7 +1430,6 @@ void seird_destroy(seird_ctx* ctx) {
   if (ctx->h_scal) cudaFreeHost(ctx->h_scal);
   if (ctx->h_cyc) cudaFreeHost(ctx->h_cyc);
   if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
-  if (ctx->h_err) cudaFreeHost(ctx->h_err);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
 }
@@ -1520,18 +1518,18 @@ static int create_impl(seird_ctx* ctx, const seird_mesh* mesh, const seird_param
   TRY(dalloc(ctx, &ctx->partial, npart));
   TRY(dalloc(ctx, &ctx->hcol, 2 * NV_STRIDE));
   TRY(dalloc(ctx, &ctx->gm, (size_t)(R + 1) * R + 2 * R + (R + 1) + R));
-  TRY(dalloc(ctx, &ctx->scal, 16));
-  TRY(dalloc(ctx, &ctx->err, 1));
-  CK(cudaMemset(ctx->err, 0, sizeof(int32_t)));
+  TRY(dalloc(ctx, &ctx->scal, SCAL_COUNT));
+  CK(cudaMemset(ctx->scal, 0, sizeof(double) * SCAL_COUNT));
+  ctx->err = reinterpret_cast<int32_t*>(ctx->scal + SCAL_ERR);
   CK(cudaMemset(ctx->U, 0, sizeof(double) * len));
   CK(cudaMemset(ctx->gm, 0, sizeof(double) * ((size_t)(R + 1) * R + 2 * R + (R + 1) + R)));
-  CK(cudaMallocHost((void**)&ctx->h_scal, sizeof(double) * 16));
+  CK(cudaMallocHost((void**)&ctx->h_scal, sizeof(double) * SCAL_COUNT));
+  std::memset(ctx->h_scal, 0, sizeof(double) * SCAL_COUNT);
+  ctx->h_err = reinterpret_cast<int32_t*>(ctx->h_scal + SCAL_ERR);
   if (o.graph) {
     TRY(dalloc(ctx, &ctx->cyc_ctl, 4));
     CK(cudaMallocHost((void**)&ctx->h_cyc, sizeof(int) * 8));
   }
-  CK(cudaMallocHost((void**)&ctx->h_err, sizeof(int32_t)));
-  *ctx->h_err = 0;
   TRY(dalloc(ctx, &ctx->dflag, 1));
   CK(cudaMallocHost((void**)&ctx->h_flag, sizeof(int)));
   // RAS
@@ -1827,8 +1825,13 @@ int seird_get_info(const seird_ctx* ctx, seird_info* info) {
 int seird_eval_residual(seird_ctx* ctx, const double* u, const double* u_prev, double* F, int on_device) {
   return host_guard(ctx, [&]() -> int {
     if (!ctx || !u || !u_prev || !F) return fail(ctx, SEIRD_EINVAL, "NULL argument");
-    TRY(to_internal(ctx, u, on_device, ctx->Ut));
-    TRY(to_internal(ctx, u_prev, on_device, ctx->stage2));
+    if (on_device) {
+      launch_gather5(ctx->hs.n, ctx->perm, u, ctx->Ut, ctx->stream, u_prev, ctx->stage2);
+      CK(cudaGetLastError());
+    } else {
+      TRY(to_internal(ctx, u, on_device, ctx->Ut));
+      TRY(to_internal(ctx, u_prev, on_device, ctx->stage2));
+    }
     double fn;
     TRY(residual(ctx, ctx->Ut, ctx->stage2, ctx->Ft, &fn));
     return from_internal(ctx, ctx->Ft, F, on_device);
