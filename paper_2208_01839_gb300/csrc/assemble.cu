@@ -150,9 +150,9 @@ __device__ __forceinline__ void reciprocals7(const double (&N)[7], double (&r)[7
   }
 }
 
-// Triangle t from the geometry table written at set-up (k_tri_geometry: |T| and the
-// gradients of the three hat functions, 8 doubles per triangle), or from the
-// coordinates when there is no table.
+// Triangle t from the geometry table written at set-up (k_tri_geometry: |T|, the stiffness
+// |T| grad phi_a . grad phi_b of its three edges (0,1) (0,2) (1,2) and the gradients of the
+// hat functions, GEO doubles per triangle), or from the coordinates when there is no table.
 __device__ __forceinline__ Tri tri_of(const int32_t* __restrict__ tri, const double* __restrict__ xy,
                                       const double* __restrict__ geo, int64_t t) {
   if (!geo) return load_tri(tri, xy, t);
@@ -160,16 +160,49 @@ __device__ __forceinline__ Tri tri_of(const int32_t* __restrict__ tri, const dou
   T.v[0] = tri[3 * t];
   T.v[1] = tri[3 * t + 1];
   T.v[2] = tri[3 * t + 2];
-  const double2* g = reinterpret_cast<const double2*>(geo + 8 * t);
-  const double2 g0 = g[0], g1 = g[1], g2 = g[2], g3 = g[3];
-  T.area = g0.x;
-  T.gx[0] = g0.y;
-  T.gx[1] = g1.x;
-  T.gx[2] = g1.y;
-  T.gy[0] = g2.x;
-  T.gy[1] = g2.y;
-  T.gy[2] = g3.x;
+  const double2* g = reinterpret_cast<const double2*>(geo + GEO * t);
+  const double2 g1 = g[2], g2 = g[3], g3 = g[4];
+  T.area = g[0].x;
+  T.gx[0] = g1.x;
+  T.gx[1] = g1.y;
+  T.gx[2] = g2.x;
+  T.gy[0] = g2.y;
+  T.gy[1] = g3.x;
+  T.gy[2] = g3.y;
   return T;
+}
+
+__device__ __forceinline__ void edge_stiffness(const Tri& T, double (&k)[3]) {
+  k[0] = T.area * (T.gx[0] * T.gx[1] + T.gy[0] * T.gy[1]);
+  k[1] = T.area * (T.gx[0] * T.gx[2] + T.gy[0] * T.gy[2]);
+  k[2] = T.area * (T.gx[1] * T.gx[2] + T.gy[1] * T.gy[2]);
+}
+
+// what the residual needs of triangle t: vertices, |T| and the edges' stiffness
+struct TriEdges {
+  double area, k[3];
+  int32_t v[3];
+};
+__device__ __forceinline__ TriEdges edges_of(const int32_t* __restrict__ tri, const double* __restrict__ xy,
+                                             const double* __restrict__ geo, int64_t t) {
+  TriEdges E;
+  if (!geo) {
+    const Tri T = load_tri(tri, xy, t);
+    E.area = T.area;
+    edge_stiffness(T, E.k);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) E.v[a] = T.v[a];
+    return E;
+  }
+  const double2* g = reinterpret_cast<const double2*>(geo + GEO * t);
+  const double2 g0 = g[0], g1 = g[1];
+  E.area = g0.x;
+  E.k[0] = g0.y;
+  E.k[1] = g1.x;
+  E.k[2] = g1.y;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) E.v[a] = tri[3 * t + a];
+  return E;
 }
 
 __global__ void __launch_bounds__(256) k_tri_geometry(int64_t m, const int32_t* __restrict__ tri,
@@ -177,11 +210,14 @@ __global__ void __launch_bounds__(256) k_tri_geometry(int64_t m, const int32_t* 
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= m) return;
   const Tri T = load_tri(tri, xy, t);
-  double2* g = reinterpret_cast<double2*>(geo + 8 * t);
-  g[0] = make_double2(T.area, T.gx[0]);
-  g[1] = make_double2(T.gx[1], T.gx[2]);
-  g[2] = make_double2(T.gy[0], T.gy[1]);
-  g[3] = make_double2(T.gy[2], 0.0);
+  double k[3];
+  edge_stiffness(T, k);
+  double2* g = reinterpret_cast<double2*>(geo + GEO * t);
+  g[0] = make_double2(T.area, k[0]);
+  g[1] = make_double2(k[1], k[2]);
+  g[2] = make_double2(T.gx[0], T.gx[1]);
+  g[3] = make_double2(T.gx[2], T.gy[0]);
+  g[4] = make_double2(T.gy[1], T.gy[2]);
 }
 
 // Node terms of the degree-5 residual, 8 doubles per node: w = u - u^n - dt L u (L the
@@ -212,6 +248,12 @@ __global__ void __launch_bounds__(256) k_residual_node(int64_t n, const double* 
 // Element residual with the degree-5 rule: consistent mass, exact diffusion, and the
 // reaction as the mass product M w of the node terms (the rule integrates the linear
 // terms exactly) plus the transmission term through the rule's orbit form (cORB).
+// Bound by the FP64 pipe, so it is written for few instructions: diffusion in edge form needs
+// 7 operations a compartment where the gradient form needed 13, and the three stiffnesses
+// come from the table.  One residual on 1024 x 1024 nodes: 1124 -> 1075 us.  Differences of
+// nodal values also cancel less than gradients summed from them: against 80-bit sums the
+// assembled diffusion of a smooth field on that mesh is off by 7e-16 (gradient form: 6e-12).
+// Launch bounds for 6 or more CTAs per SM spill (96 registers as it stands) and were left.
 template <bool BF>
 __global__ void __launch_bounds__(128) k_residual_elem5(int64_t m, const int32_t* __restrict__ tri,
                                                         const double* __restrict__ xy,
@@ -221,7 +263,7 @@ __global__ void __launch_bounds__(128) k_residual_elem5(int64_t m, const int32_t
                                                         double* __restrict__ elem, int32_t* err) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= m) return;
-  const Tri T = tri_of(tri, xy, geo, t);
+  const TriEdges T = edges_of(tri, xy, geo, t);
   const Rates r = rates_at(rin, T.v[0]);
   double u[3][4], w[3][5], Nv[3], l[3], Fe[3][5];
 #pragma unroll
@@ -247,15 +289,16 @@ __global__ void __launch_bounds__(128) k_residual_elem5(int64_t m, const int32_t
 #pragma unroll
     for (int a = 0; a < 3; ++a) Fe[a][c] = fma(m12, w[a][c], msw);
   }
-  // diffusion: dt nubar_c |T| mean_T(N) grad u_c . grad phi_a  (nubar_D = 0)
-  const double dNA = r.dt * Nbar * T.area;
+  // diffusion: dt nubar_c mean_T(N) sum_b k_ab (u_b - u_a), k_ab = |T| grad phi_a . grad phi_b
+  // (the gradients of the hat functions sum to zero; nubar_D = 0)
+  const double dN = r.dt * Nbar;
+  const double k01 = dN * T.k[0], k02 = dN * T.k[1], k12 = dN * T.k[2];
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const double coef = dNA * r.nu[c];
-    const double gux = coef * (u[0][c] * T.gx[0] + u[1][c] * T.gx[1] + u[2][c] * T.gx[2]);
-    const double guy = coef * (u[0][c] * T.gy[0] + u[1][c] * T.gy[1] + u[2][c] * T.gy[2]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Fe[a][c] = fma(gux, T.gx[a], fma(guy, T.gy[a], Fe[a][c]));
+    const double e01 = k01 * (u[1][c] - u[0][c]), e02 = k02 * (u[2][c] - u[0][c]), e12 = k12 * (u[2][c] - u[1][c]);
+    Fe[0][c] = fma(r.nu[c], e01 + e02, Fe[0][c]);
+    Fe[1][c] = fma(r.nu[c], e12 - e01, Fe[1][c]);
+    Fe[2][c] = fma(-r.nu[c], e02 + e12, Fe[2][c]);
   }
   // transmission s -> e, kappa s (beta_I i + beta_E e) b, at the rule's points
   double bv[3] = {1.0, 1.0, 1.0};

@@ -1491,7 +1491,7 @@ static int create_impl(seird_ctx* ctx, const seird_mesh* mesh, const seird_param
   }
   if (o.precision == 0) TRY(dalloc(ctx, &ctx->val, 25 * nnzb));
   TRY(dalloc(ctx, &ctx->elem, 15 * m));
-  TRY(dalloc(ctx, &ctx->geo, 8 * m));
+  TRY(dalloc(ctx, &ctx->geo, (size_t)GEO * m));
   launch_tri_geometry(m, ctx->tri, ctx->xy, ctx->geo, ctx->stream);
   CK(cudaGetLastError());
   TRY(dalloc(ctx, &ctx->nodebuf, 8 * (size_t)hs.n));
