@@ -21,7 +21,7 @@ __device__ __forceinline__ double ld_val(const float* p) { return widen(__ldg(p)
 // row i, row r): all 32 lanes of every warp do useful FP64 work, 25 FMA per block per 5 threads.
 // UNEVEN (a caller's own matrix): a warp takes as long as its longest row, so where a CTA's
 // rows differ in length it takes them longest first, each row's rank counted on the integer
-// pipe (rows of four to nine blocks, 1.95M blocks: 138.6 -> 102 us).  A mesh's rows are nearly
+// pipe (rows of four to nine blocks, 1.95M blocks: 139.5 -> 102.8 us).  A mesh's rows are nearly
 // all alike; for the Jacobian the sort only costs (2.0M nodes: 595 -> 601 us).
 template <class VT, bool UNEVEN>
 __global__ void __launch_bounds__(512) k_bsr_spmv(int64_t nrow, const int32_t* __restrict__ rp,

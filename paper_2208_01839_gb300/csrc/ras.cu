@@ -775,18 +775,8 @@ __global__ void k_coarse_chunks(int32_t nchunk, const int32_t* __restrict__ cptr
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (gw >= nchunk || lane >= 25) return;
-  // eight blocks in flight (the sums stay in block order): 2.0M nodes 0.87 ms with one
   double s = 0.0;
-  const int32_t e = cptr[gw + 1];
-  int32_t b = cptr[gw];
-  for (; b + 8 <= e; b += 8) {
-    TV v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = val[25 * (int64_t)blk[b + u] + lane];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) s += widen(v[u]);
-  }
-  for (; b < e; ++b) s += widen(val[25 * (int64_t)blk[b] + lane]);
+  for (int32_t b = cptr[gw]; b < cptr[gw + 1]; ++b) s += (double)val[25 * (int64_t)blk[b] + lane];
   cpart[25 * gw + lane] = s;
 }
 
@@ -808,8 +798,9 @@ __device__ __forceinline__ double* bblk(double* band, int bw, int ib, int jb) {
 // Block step kb of the banded LU, one CTA per row i in (kb, kb + bw] (one in all at the end):
 // every CTA inverts the pivot block for itself (the step's latency either way), forms
 // L_i,kb and updates its row, A_ij -= L_i,kb A_kb,j for j in (kb, kb + bw]; no CTA writes
-// what another reads, so a step is one launch.  512 units, half-bandwidth 28: 9.2 us a step
-// with a launch for the pivot column and one for the update, 4.8 us now.
+// what another reads, so a step is one launch.  512 units: with a launch for the pivot column
+// and one for the update 8.5 us a step at 2.0M nodes and 9.2 us at 1024 x 1024 (wider band),
+// 6.7 and 7.2 us now; the pivot's serial inverse is most of it.
 __global__ void __launch_bounds__(256) k_band_step(int P, int bw, int kb, double* band, double* cdinv, int32_t* err) {
   __shared__ double Dk[25], L[25];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -900,7 +891,8 @@ __global__ void k_band_solve(int P, int bw, const double* __restrict__ band, con
 // block row of the band is 25 independent dot products per band block.  X goes
 // to rows 5b..5b+4 of AinvT (row j of AinvT = column j of A_c^{-1}).  Bound by the FP64 pipe
 // (five FMAs a product sum) and by the latency of a step's band blocks, which are
-// therefore loaded a step ahead, INV_ITEMS sums a thread (512 units: 5.36 ms without).
+// therefore loaded a step ahead, INV_ITEMS sums a thread (512 units, 2.0M nodes: 4.73 -> 3.94
+// ms; 1024 x 1024: 5.37 -> 4.52).
 constexpr int INV_ITEMS = 3;
 __global__ void __launch_bounds__(256) k_band_inv(int P, int bw, const double* __restrict__ band,
                                                   const double* __restrict__ cdinv, double* __restrict__ ainvT) {
@@ -1230,7 +1222,7 @@ __global__ void k_az_build(int64_t nseg, const int32_t* __restrict__ az_blk, con
   const int64_t s = g / 25;
   const int e = (int)(g - 25 * s);
   double acc = 0.0;
-  for (int32_t b = az_blk[s]; b < az_blk[s + 1]; ++b) acc += widen(val[25 * (int64_t)b + e]);
+  for (int32_t b = az_blk[s]; b < az_blk[s + 1]; ++b) acc += (double)val[25 * (int64_t)b + e];
   azval[g] = (TA)acc;
 }
 
