@@ -489,23 +489,10 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
                                                     const double* __restrict__ bfield, Rates rin,
                                                     T* __restrict__ rec, int32_t* err) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  // A, beta_I, beta_E, dt, nubar_S..R in type T (see rate_consts)
-  constexpr bool kCTA = sizeof(T) == 4;
-  __shared__ T srk[8];
-  if (kCTA && !rin.tab) {
-    if (threadIdx.x == 0) {
-      srk[0] = (T)rin.A;
-      srk[1] = (T)rin.bi;
-      srk[2] = (T)rin.be;
-      srk[3] = (T)rin.dt;
-      for (int c = 0; c < 4; ++c) srk[4 + c] = (T)rin.nu[c];
-    }
-    __syncthreads();
-  }
   if (t >= m) return;
   const Tri Tg = tri_of(tri, xy, geo, t);
   const Rates r = rates_at(rin, Tg.v[0]);
-  const bool shr = kCTA && !rin.tab;
+  const bool f32 = sizeof(T) == 4 && !rin.tab;  // the rates as the host rounded them (see rate_consts)
   TriT<T> Tt;
   Tt.area = (T)Tg.area;
 #pragma unroll
@@ -526,7 +513,7 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
   out[0] = Tt.area;
   // N-weighted stiffness dt |T| mean(N) grad phi_a . grad phi_b
   // the gather reads the sums below already scaled: K and P by dt, G_c by dt nu_c
-  const T dtT = shr ? srk[3] : (T)r.dt;
+  const T dtT = f32 ? (T)rin.f[0] : (T)r.dt;
   const T an = dtT * Tt.area * Nbar;
   out[REC_K + 0] = an * (Tt.gx[0] * Tt.gx[0] + Tt.gy[0] * Tt.gy[0]);
   out[REC_K + 1] = an * (Tt.gx[1] * Tt.gx[1] + Tt.gy[1] * Tt.gy[1]);
@@ -541,7 +528,7 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
     for (int c = 0; c < 4; ++c) {
       const T gux = u[0][c] * Tt.gx[0] + u[1][c] * Tt.gx[1] + u[2][c] * Tt.gx[2];
       const T guy = u[0][c] * Tt.gy[0] + u[1][c] * Tt.gy[1] + u[2][c] * Tt.gy[2];
-      const T gsc = a3 * dtT * (shr ? srk[4 + c] : (T)r.nu[c]);
+      const T gsc = a3 * dtT * (f32 ? (T)rin.f[1 + c] : (T)r.nu[c]);
       const T gxs = gsc * gux, gys = gsc * guy;
 #pragma unroll
       for (int a = 0; a < 3; ++a) out[REC_G + 4 * a + c] = gxs * Tt.gx[a] + gys * Tt.gy[a];
@@ -561,7 +548,7 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
 #pragma unroll
     for (int a = 0; a < 3; ++a) bv[a] = (T)bfield[Tt.v[a]];
   }
-  const T A = shr ? srk[0] : (T)r.A, bi = shr ? srk[1] : (T)r.bi, be = shr ? srk[2] : (T)r.be;
+  const T A = f32 ? (T)rin.f[13] : (T)r.A, bi = f32 ? (T)rin.f[14] : (T)r.bi, be = f32 ? (T)rin.f[15] : (T)r.be;
   bool bad = false;
   if (RULE == 0 && !PIC) {
     // the degree-5 rule by its orbits (cORB): per moment, the centroid value, the two
@@ -673,32 +660,28 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
 }
 
 // dt, nubar_S..R, alpha, mu, sigma, gamma_E, gamma_R, gamma_D and the two sums of rates out of
-// E and I in type T.  FP32 kernels with one
-// set of rates (no per-sample table) convert them once per CTA: GB300 converts FP64 to FP32
-// at its FP64 rate, which per thread would cost as much as the block's arithmetic.  Every
-// thread of the CTA calls it.
+// E and I in type T.  FP32 kernels with one set of rates (no per-sample table) take them as
+// the host rounded them, straight from the kernel's parameters: GB300 converts FP64 to FP32 at
+// its FP64 rate, and values that one thread converts and the CTA reads from shared memory
+// cost a load each in every thread (1024 x 1024 nodes: gather 331 us with 11 of them, 346 with
+// 13, 329 this way; record 461 -> 457).
 template <class T>
 __device__ __forceinline__ void rate_consts(const Rates& rin, const Rates& r, T (&k)[13]) {
-  auto fill = [](const Rates& q, T* o) {
-    o[0] = (T)q.dt;
-    for (int c = 0; c < 4; ++c) o[1 + c] = (T)q.nu[c];
-    o[5] = (T)q.alpha;
-    o[6] = (T)q.mu;
-    o[7] = (T)q.sigma;
-    o[8] = (T)q.ge;
-    o[9] = (T)q.gr;
-    o[10] = (T)q.gd;
-    o[11] = (T)q.out_e;
-    o[12] = (T)q.out_i;
-  };
   if (sizeof(T) == 4 && !rin.tab) {
-    __shared__ T sk[13];
-    if (threadIdx.x == 0) fill(rin, sk);
-    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 13; ++i) k[i] = sk[i];
+    for (int i = 0; i < 13; ++i) k[i] = rin.f[i];
   } else {
-    fill(r, k);
+    k[0] = (T)r.dt;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) k[1 + c] = (T)r.nu[c];
+    k[5] = (T)r.alpha;
+    k[6] = (T)r.mu;
+    k[7] = (T)r.sigma;
+    k[8] = (T)r.ge;
+    k[9] = (T)r.gr;
+    k[10] = (T)r.gd;
+    k[11] = (T)r.out_e;
+    k[12] = (T)r.out_i;
   }
 }
 
@@ -787,7 +770,8 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
   const T nu0 = rk[1], nu1 = rk[2], nu2 = rk[3], nu3 = rk[4];
   const T dMr = dt * Mr;
   const T alpha = rk[5], mu = rk[6], sigma = rk[7], ge = rk[8], gr = rk[9], gd = rk[10], outE = rk[11], outI = rk[12];
-  const bool births = alpha != T(0), deaths = mu != T(0);  // both zero in the paper's runs: no products then
+  // both zero in the paper's runs: no FP64 products then
+  const bool births = sizeof(T) == 4 || alpha != T(0), deaths = sizeof(T) == 4 || mu != T(0);
   T B[5][5];
 #pragma unroll
   for (int i = 0; i < 5; ++i)
