@@ -90,7 +90,7 @@ struct HostSetup {
     std::vector<int64_t> src;     // [nblocks] factor block (>= 0) or -1-R for the inverted pivot of row R
     std::vector<int32_t> col;     // [nblocks] sweep position of the entry each block multiplies, -1 - position for an
                                   // entry that has left the window; pivots (0) multiply the row's own first value
-    std::vector<int32_t> brow;    // [nblocks] row R (absolute) of each block
+    std::vector<int32_t> brow;    // [nblocks] row R (absolute) of each block (forward plan only)
     std::vector<int32_t> info;    // [NL][4] per position: forward (node, first block in its stage, blocks, backward
                                   // position), backward (forward position, first block, blocks, node if owned else -1)
   } sp_fwd, sp_bwd;

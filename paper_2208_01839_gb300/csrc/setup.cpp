@@ -543,18 +543,23 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
         std::vector<int32_t>& order = S.order[dir];
         order.resize(nl);
         std::vector<int32_t> fill(lb.begin(), lb.end() - 1);
-        if (dir == 0) {
-          for (int32_t i = 0; i < nl; ++i) order[fill[lev[i]]++] = i;
-        } else {
-          for (int32_t i = nl - 1; i >= 0; --i) order[fill[lev[i]]++] = i;
-        }
         // the rows of a level are independent: longest first, so that rows of about the same
-        // length share a warp in the factorisation and the solves
-        for (int32_t i = 0; i < nl; ++i)
+        // length share a warp in the factorisation and the solves (rows dealt to their levels
+        // in descending length, equal lengths in sweep order: two counting passes)
+        int32_t most = 0;
+        for (int32_t i = 0; i < nl; ++i) {
           cnt[i] = (int32_t)(dir == 0 ? S.diag[i] - rstart[i] : rstart[i + 1] - S.diag[i] - 1);
-        for (int32_t v = 0; v < nlev; ++v)
-          std::stable_sort(order.begin() + lb[v], order.begin() + lb[v + 1],
-                           [&](int32_t a, int32_t b) { return cnt[a] > cnt[b]; });
+          most = std::max(most, cnt[i]);
+        }
+        std::vector<int32_t> at(most + 2, 0), byLength(nl);
+        for (int32_t i = 0; i < nl; ++i) ++at[most - cnt[i] + 1];
+        for (int32_t c = 0; c <= most; ++c) at[c + 1] += at[c];
+        if (dir == 0) {
+          for (int32_t i = 0; i < nl; ++i) byLength[at[most - cnt[i]]++] = i;
+        } else {
+          for (int32_t i = nl - 1; i >= 0; --i) byLength[at[most - cnt[i]]++] = i;
+        }
+        for (int32_t k = 0; k < nl; ++k) order[fill[lev[byLength[k]]]++] = byLength[k];
       }
       for (int32_t l = 0; l < nl; ++l) loc[nodes[l]] = -1;
     });
@@ -703,7 +708,7 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
               T.col.push_back(posb[hs.l_col[a]]);
             }
           }
-          T.brow.resize(T.src.size(), (int32_t)R);
+          if (dir == 0) T.brow.resize(T.src.size(), (int32_t)R);
           in_level += nb;
           ++pos;
         }
@@ -726,7 +731,7 @@ int build_setup(const seird_mesh* mesh, const seird_options* opt, HostSetup& hs,
     sp.info.resize(4 * (size_t)hs.sd_row0[P]);
     sp.src.resize(soff[P]);
     sp.col.resize(soff[P]);
-    sp.brow.resize(soff[P]);
+    if (dir == 0) sp.brow.resize(soff[P]);
     parallel_for(P, setup_threads(P), [&](int32_t q, int) {
       PlanPart& T = pp[q];
       const int64_t l0 = loff[q], r0 = hs.sd_row0[q], s0 = soff[q];
@@ -1047,7 +1052,7 @@ int64_t check_setup(const HostSetup& hs, std::string& first) {
             owned += own;
           }
           fail(rec[2] == expect, "row block count");
-          for (int32_t j = 0; j < rec[2]; ++j) fail(sp.brow[b0 + rec[1] + j] == R, "factor block of another row");
+          for (int32_t j = 0; dir == 0 && j < rec[2]; ++j) fail(sp.brow[b0 + rec[1] + j] == R, "factor block of another row");
           for (int32_t j = dir == 0 ? 1 : 0; j < rec[2]; ++j) {
             const int32_t c = sp.col[b0 + rec[1] + j], pos = c < 0 ? -1 - c : c;
             fail(pos >= 0 && pos < k0, "dependency not in an earlier stage");
