@@ -150,13 +150,13 @@ typedef struct {
                              ||F(u^n)|| either way.  Each degree keeps one more state (5n doubles) (0) */
   int32_t autotune;       /* 1: at the first linear solve, time the candidate launch shapes of the SpMV
                              (128/256/512 threads per CTA), of the Gram-Schmidt kernels (2/3/4/6 CTAs
-                             per SM, 128- or 256-entry tiles) and of the subdomain solves (1-4 blocks of
-                             solution entries loaded per batch, 7 or 3 consumer warps per CTA, a factor
-                             ring of two stages or one) on the context's own vectors and factors
+                             per SM, 128- or 256-entry tiles) and of the subdomain solves (CTAs of 256 or
+                             160 threads, a factor ring of several stages or one) on the context's own
+                             vectors and factors
                              and keep the fastest; the choice is reported by seird_get_info.  The
                              Gram-Schmidt shape sets the order of its sums, so results are reproducible
                              for a given choice, not across choices; the other choices leave every sum
-                             unchanged.  0: fixed shapes (256 threads, 3 CTAs per SM, 256, 2 blocks) (0) */
+                             unchanged.  0: fixed shapes (256 threads, 3 CTAs per SM, 256, the larger solve shapes) (0) */
   int32_t graph;          /* 1: each GMRES restart cycle runs as one replay of a CUDA graph captured at
                              the first solve: iteration j is a conditional node that the Givens kernel
                              of iteration j - 1 arms while the residual estimate is above the
@@ -225,11 +225,13 @@ typedef struct {
   int32_t coarse_units;        /* units of the coarse space (groups of options.coarse_group subdomains) */
   int32_t spmv_threads;        /* launch shapes in use (options.autotune): SpMV threads per CTA, */
   int32_t cgs_ctas;            /* Gram-Schmidt CTAs, */
-  int32_t cgs_tile;            /* Gram-Schmidt tile entries (0: 256 up to depth 27, then 128) */
-  int32_t ilu_batch;           /* subdomain solves: blocks whose solution entries a row loads before
-                                  their FMAs (1-4), */
-  int32_t ilu_warps;           /* consumer warps per subdomain CTA (7, or 3 in CTAs of 128 threads), */
-  int32_t ilu_ring;            /* and factor blocks in the shared-memory ring (236: two stages, 118: one) */
+  int32_t cgs_tile;            /* Gram-Schmidt tile entries (0: 256 up to depth 27, then 128; 64 on
+                                  vectors too short to give every SM a tile) */
+  int32_t ilu_batch;           /* kept for callers that set it; the subdomain solves no longer load
+                                  solution entries in batches, so it selects nothing (1-4), */
+  int32_t ilu_warps;           /* subdomain CTAs: 7 (256 threads, six warps on rows) or 3 (160, three), */
+  int32_t ilu_ring;            /* factor ring in shared memory: 236 (several stages, as many blocks as the
+                                  CTAs that share an SM leave room for) or 118 (one stage) */
 } seird_info;
 
 typedef struct seird_ctx seird_ctx;
@@ -383,8 +385,9 @@ int seird_precond_apply(seird_ctx* ctx, const double* r, double* z, int on_devic
 
 /* Pins launch shapes (each 0 keeps the current one): SpMV threads per CTA (128, 256,
  * 512), Gram-Schmidt CTAs (1 .. 64 x SMs) and tile entries (128, 256), and the
- * subdomain solves' dependency-load batch (1-4 blocks), consumer warps (7 or 3)
- * and factor-ring size (236 or 118 blocks; 118 only when every stage fits it).  The autotuner
+ * subdomain solves' batch (1-4; checked and reported, selects nothing), CTA form (7: 256
+ * threads, 3: 160) and factor ring (236: several stages, 118: one; 118 only when every
+ * stage fits it).  The autotuner
  * (options.autotune) does not change shapes pinned this way, so the shapes one
  * run reported by seird_get_info reproduce its sums in another run (the
  * Gram-Schmidt shape sets the order of its sums; the other shapes do not change
