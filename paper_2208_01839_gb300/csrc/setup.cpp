@@ -1028,9 +1028,10 @@ int64_t check_setup(const HostSetup& hs, std::string& first) {
       for (int32_t v = v0; v < v1 && !bad; ++v) {
         const int32_t k0 = sp.levpos[v], k1 = sp.levpos[v + 1];
         const int64_t b0 = sp.levblk[v], nbs = sp.levblk[v + 1] - b0;
-        // (a forward row holds its inverted pivot besides its lower blocks)
-        fail(k1 >= k0 && k1 - k0 <= SOLVE_BUF_ROWS && nbs >= 0 && nbs <= SOLVE_BUF_BLOCKS + (dir == 0 && k1 - k0 == 1),
-             "stage exceeds the rings");
+        // a forward row holds its inverted pivot besides its lower blocks; a row alone in its backward
+        // stage counts its pivot too, as the limit of the one-stage ring does (max_row_blocks)
+        const int64_t most = SOLVE_BUF_BLOCKS + (k1 - k0 == 1 ? (dir == 0 ? 1 : -1) : 0);
+        fail(k1 >= k0 && k1 - k0 <= SOLVE_BUF_ROWS && nbs >= 0 && nbs <= most, "stage exceeds the rings");
         const int4 st = sp.stage[v];
         fail(st.x == k0 && st.y == b0 && stage_rows(st) == k1 - k0 && stage_blocks(st) == nbs, "stage record");
         for (int32_t k = k0; k < k1; ++k) {

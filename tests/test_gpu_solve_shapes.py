@@ -79,6 +79,21 @@ def _wheel_strip(spokes, cells):
     return np.concatenate(xy), np.concatenate([np.array(tri), stri + off]).astype(np.int32)
 
 
+@pytest.mark.parametrize("spokes,hub_last,accepted", [(117, False, True), (118, False, False),
+                                                      (118, True, True), (119, True, False)])
+def test_longest_row_of_the_one_stage_ring(spokes, hub_last, accepted):
+    """118 blocks in a row's sweep: its lower ones, or its pivot and its upper ones."""
+    xy, tri = _wheel_strip(spokes, 40)
+    if hub_last:
+        xy, tri = xy[::-1].copy(), (len(xy) - 1 - tri).astype(np.int32)
+    check = functools.partial(S.setup_check, xy, tri, owner=np.zeros(len(xy), dtype=np.int32), overlap=0, ilu_fill=1)
+    if accepted:
+        assert check()["violations"] == 0
+    else:
+        with pytest.raises(S.SeirdError, match="stage exceeds the rings"):
+            check()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("spokes", [5, 30, 31, 32, 33, 40, 100])
