@@ -466,9 +466,6 @@ __global__ void k_sum_partials(int64_t np, const double* __restrict__ partial, d
   }
 }
 
-__device__ __forceinline__ double fmaR(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float fmaR(float a, float b, float c) { return fmaf(a, b, c); }
-
 // symmetric pair index: (0,0) (1,1) (2,2) (0,1) (0,2) (1,2)
 __device__ __forceinline__ int sym(int a, int b) {
   return a == b ? a : (a + b + 2);
@@ -477,7 +474,11 @@ __device__ __forceinline__ int sym(int a, int b) {
 // Jacobian record of a triangle.  FP64: bound by the FP64 pipe (200k nodes: 296 us with four
 // moments and the mean density summed apart, record and gather together 540 -> 474 us).
 // T is the arithmetic and storage type: FP64, or FP32 when the Jacobian only
-// feeds the FP32 operator and FP32 factors of the mixed-precision path.
+// feeds the FP32 operator and FP32 factors of the mixed-precision path.  In FP32 the order
+// of the sums and products is part of the result: a caller reads the FP32 matrix and its
+// products in FP64, where another order shows at 1e-7, and the FP64 form's fewer operations
+// do not make it faster (record and gather on 1024 x 1024 nodes: 785 us with them, 782
+// without).  So each precision has its own form.
 // PIC: the record of the Picard matrix of Eq. weak_vec_implicit instead (no
 // derivative of N in the diffusion coefficient, and moment 0 holds the
 // coefficient kappa beta_I i b of B(u)'s (E, S) entry instead of the Allee
@@ -489,10 +490,23 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
                                                     const double* __restrict__ bfield, Rates rin,
                                                     T* __restrict__ rec, int32_t* err) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  // A, beta_I, beta_E, dt, nubar_S..R in type T (see rate_consts)
+  constexpr bool F32 = sizeof(T) == 4;
+  __shared__ T srk[8];
+  if (F32 && !rin.tab) {
+    if (threadIdx.x == 0) {
+      srk[0] = (T)rin.A;
+      srk[1] = (T)rin.bi;
+      srk[2] = (T)rin.be;
+      srk[3] = (T)rin.dt;
+      for (int c = 0; c < 4; ++c) srk[4 + c] = (T)rin.nu[c];
+    }
+    __syncthreads();
+  }
   if (t >= m) return;
   const Tri Tg = tri_of(tri, xy, geo, t);
   const Rates r = rates_at(rin, Tg.v[0]);
-  const bool f32 = sizeof(T) == 4 && !rin.tab;  // the rates as the host rounded them (see rate_consts)
+  const bool shr = F32 && !rin.tab;
   TriT<T> Tt;
   Tt.area = (T)Tg.area;
 #pragma unroll
@@ -501,19 +515,23 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
     Tt.gy[a] = (T)Tg.gy[a];
     Tt.v[a] = Tg.v[a];
   }
-  T u[3][5], Nv[3];
+  T u[3][5], Nv[3], Nsum = T(0);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
 #pragma unroll
-    for (int c = 0; c < 5; ++c) u[a][c] = (T)U[5 * (int64_t)Tt.v[a] + c];
+    for (int c = 0; c < 5; ++c) {
+      u[a][c] = (T)U[5 * (int64_t)Tt.v[a] + c];
+      if (F32) Nsum += u[a][c];
+    }
     Nv[a] = u[a][0] + u[a][1] + u[a][2] + u[a][3] + u[a][4];
   }
-  const T Nbar = (Nv[0] + Nv[1] + Nv[2]) * T(1.0 / 3.0);
+  if (!F32) Nsum = Nv[0] + Nv[1] + Nv[2];
+  const T Nbar = Nsum * T(1.0 / 3.0);
   T* out = rec + (int64_t)REC * t;
   out[0] = Tt.area;
   // N-weighted stiffness dt |T| mean(N) grad phi_a . grad phi_b
   // the gather reads the sums below already scaled: K and P by dt, G_c by dt nu_c
-  const T dtT = f32 ? (T)rin.f[0] : (T)r.dt;
+  const T dtT = shr ? srk[3] : (T)r.dt;
   const T an = dtT * Tt.area * Nbar;
   out[REC_K + 0] = an * (Tt.gx[0] * Tt.gx[0] + Tt.gy[0] * Tt.gy[0]);
   out[REC_K + 1] = an * (Tt.gx[1] * Tt.gx[1] + Tt.gy[1] * Tt.gy[1]);
@@ -528,19 +546,21 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
     for (int c = 0; c < 4; ++c) {
       const T gux = u[0][c] * Tt.gx[0] + u[1][c] * Tt.gx[1] + u[2][c] * Tt.gx[2];
       const T guy = u[0][c] * Tt.gy[0] + u[1][c] * Tt.gy[1] + u[2][c] * Tt.gy[2];
-      const T gsc = a3 * dtT * (f32 ? (T)rin.f[1 + c] : (T)r.nu[c]);
+      const T gsc = a3 * dtT * (shr ? srk[4 + c] : (T)r.nu[c]);
       const T gxs = gsc * gux, gys = gsc * guy;
 #pragma unroll
-      for (int a = 0; a < 3; ++a) out[REC_G + 4 * a + c] = gxs * Tt.gx[a] + gys * Tt.gy[a];
+      for (int a = 0; a < 3; ++a)
+        out[REC_G + 4 * a + c] = F32 ? gsc * (gux * Tt.gx[a] + guy * Tt.gy[a]) : gxs * Tt.gx[a] + gys * Tt.gy[a];
     }
   }
   // reaction moments P^k_ab = dt |T| sum_q w_q phi_a phi_b rho_k(x_q):
   //   rho_0 = A s lam / N^2 (d kappa/du_c' = A/N^2 for every c'), rho_1 = kappa lam,
-  //   rho_2 = kappa s beta_E b, rho_3 = kappa s beta_I b (the moments of kappa s b times
-  // the two rates: three moments are summed, not four).
-  T P[3][6];
+  //   rho_2 = kappa s beta_E b, rho_3 = kappa s beta_I b.
+  // FP64 sums the moments of kappa s b once and multiplies them by the two rates: NM = 3.
+  constexpr int NM = F32 ? 4 : 3;
+  T P[NM][6];
 #pragma unroll
-  for (int k = 0; k < 3; ++k)
+  for (int k = 0; k < NM; ++k)
 #pragma unroll
     for (int s = 0; s < 6; ++s) P[k][s] = T(0);
   T bv[3] = {T(1), T(1), T(1)};
@@ -548,7 +568,11 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
 #pragma unroll
     for (int a = 0; a < 3; ++a) bv[a] = (T)bfield[Tt.v[a]];
   }
-  const T A = f32 ? (T)rin.f[13] : (T)r.A, bi = f32 ? (T)rin.f[14] : (T)r.bi, be = f32 ? (T)rin.f[15] : (T)r.be;
+  const T A = shr ? srk[0] : (T)r.A, bi = shr ? srk[1] : (T)r.bi, be = shr ? srk[2] : (T)r.be;
+  auto infect = [&](T ksb, T (&rho)[NM]) {  // moments 2 and 3 from kappa s b
+    rho[2] = F32 ? ksb * be : ksb;
+    if constexpr (F32) rho[3] = ksb * bi;
+  };
   bool bad = false;
   if (RULE == 0 && !PIC) {
     // the degree-5 rule by its orbits (cORB): per moment, the centroid value, the two
@@ -578,15 +602,15 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
       for (int q = 0; q < 7; ++q) rq[q] = T(1) / Nq[q];
     }
     // rho at point q from s, l, b there
-    auto moments = [&](int q, T s, T lv, T b, T (&rho)[3]) {
+    auto moments = [&](int q, T s, T lv, T b, T (&rho)[NM]) {
       const T Ar = A * rq[q];
       const T kappa = T(1) - Ar;
       const T lam = lv * b;
       rho[0] = Ar * rq[q] * (s * lam);
       rho[1] = kappa * lam;
-      rho[2] = kappa * s * b;
+      infect(kappa * s * b, rho);
     };
-    T rc[3], S1[3] = {0, 0, 0}, S2[3] = {0, 0, 0};
+    T rc[NM], S1[NM] = {}, S2[NM] = {};
     moments(0, Ss * T(1.0 / 3.0), Sl * T(1.0 / 3.0), BF ? Sb * T(1.0 / 3.0) : T(1), rc);
     // P[k][a] (a < 3, pair (a, a)) and P[k][3 + (2 - c)] (the pair opposite vertex c) take the
     // point values; the orbit sums and the centroid value are added to all pairs at the end
@@ -594,11 +618,11 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
     const T cdR1 = ar * orb<T>(14), coR1 = ar * orb<T>(16), cdR2 = ar * orb<T>(18), coR2 = ar * orb<T>(20);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      T rho1[3], rho2[3];
+      T rho1[NM], rho2[NM];
       moments(1 + k, A1 * Ss + D1 * u[k][0], A1 * Sl + D1 * l[k], BF ? A1 * Sb + D1 * bv[k] : T(1), rho1);
       moments(4 + k, A2 * Ss + D2 * u[k][0], A2 * Sl + D2 * l[k], BF ? A2 * Sb + D2 * bv[k] : T(1), rho2);
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
+      for (int j = 0; j < NM; ++j) {
         S1[j] += rho1[j];
         S2[j] += rho2[j];
         P[j][k] = cdR1 * rho1[j] + cdR2 * rho2[j];
@@ -608,7 +632,7 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
     const T c0 = ar * orb<T>(12), cdS1 = ar * orb<T>(13), coS1 = ar * orb<T>(15);
     const T cdS2 = ar * orb<T>(17), coS2 = ar * orb<T>(19);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
+    for (int j = 0; j < NM; ++j) {
       const T base = c0 * rc[j];
       const T bd = base + cdS1 * S1[j] + cdS2 * S2[j];
       const T bo = base + coS1 * S1[j] + coS2 * S2[j];
@@ -632,19 +656,19 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
       const T invN = T(1) / N;
       const T kappa = T(1) - A * invN;
       const T lam = (bi * iq + be * eq) * bq;
-      T rho[3];
+      T rho[NM];
       rho[0] = PIC ? kappa * bi * iq * bq : A * invN * invN * sq * lam;
       rho[1] = kappa * lam;
-      rho[2] = kappa * sq * bq;
+      infect(kappa * sq * bq, rho);
 #pragma unroll
       for (int s = 0; s < 6; ++s) {
         const T cw = (T)cQC[RULE][q][s];  // w_q phi_a phi_b; the area multiplies once at the end
 #pragma unroll
-        for (int k = 0; k < 3; ++k) P[k][s] += cw * rho[k];
+        for (int k = 0; k < NM; ++k) P[k][s] += cw * rho[k];
       }
     }
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < NM; ++k)
 #pragma unroll
       for (int s = 0; s < 6; ++s) P[k][s] *= dtT * Tt.area;
   }
@@ -653,35 +677,36 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
   for (int s = 0; s < 6; ++s) {
     out[REC_P + 4 * s] = P[0][s];
     out[REC_P + 4 * s + 1] = P[1][s];
-    out[REC_P + 4 * s + 2] = be * P[2][s];
-    out[REC_P + 4 * s + 3] = bi * P[2][s];
+    out[REC_P + 4 * s + 2] = F32 ? P[2][s] : be * P[2][s];
+    out[REC_P + 4 * s + 3] = F32 ? P[NM - 1][s] : bi * P[2][s];
   }
   out[REC_K + 6] = T(0);
 }
 
-// dt, nubar_S..R, alpha, mu, sigma, gamma_E, gamma_R, gamma_D and the two sums of rates out of
-// E and I in type T.  FP32 kernels with one set of rates (no per-sample table) take them as
-// the host rounded them, straight from the kernel's parameters: GB300 converts FP64 to FP32 at
-// its FP64 rate, and values that one thread converts and the CTA reads from shared memory
-// cost a load each in every thread (1024 x 1024 nodes: gather 331 us with 11 of them, 346 with
-// 13, 329 this way; record 461 -> 457).
+// dt, nubar_S..R, alpha, mu, sigma, gamma_E, gamma_R, gamma_D in type T.  FP32 kernels with one
+// set of rates (no per-sample table) convert them once per CTA: GB300 converts FP64 to FP32
+// at its FP64 rate, which per thread would cost as much as the block's arithmetic.  Every
+// thread of the CTA calls it.
 template <class T>
-__device__ __forceinline__ void rate_consts(const Rates& rin, const Rates& r, T (&k)[13]) {
+__device__ __forceinline__ void rate_consts(const Rates& rin, const Rates& r, T (&k)[11]) {
+  auto fill = [](const Rates& q, T* o) {
+    o[0] = (T)q.dt;
+    for (int c = 0; c < 4; ++c) o[1 + c] = (T)q.nu[c];
+    o[5] = (T)q.alpha;
+    o[6] = (T)q.mu;
+    o[7] = (T)q.sigma;
+    o[8] = (T)q.ge;
+    o[9] = (T)q.gr;
+    o[10] = (T)q.gd;
+  };
   if (sizeof(T) == 4 && !rin.tab) {
+    __shared__ T sk[11];
+    if (threadIdx.x == 0) fill(rin, sk);
+    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 13; ++i) k[i] = rin.f[i];
+    for (int i = 0; i < 11; ++i) k[i] = sk[i];
   } else {
-    k[0] = (T)r.dt;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) k[1 + c] = (T)r.nu[c];
-    k[5] = (T)r.alpha;
-    k[6] = (T)r.mu;
-    k[7] = (T)r.sigma;
-    k[8] = (T)r.ge;
-    k[9] = (T)r.gr;
-    k[10] = (T)r.gd;
-    k[11] = (T)r.out_e;
-    k[12] = (T)r.out_i;
+    fill(r, k);
   }
 }
 
@@ -717,6 +742,7 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
                                                     const int32_t* __restrict__ inc, const T* __restrict__ rec,
                                                     const int32_t* __restrict__ tri, Rates rin,
                                                     T* __restrict__ val) {
+  constexpr bool F32 = sizeof(T) == 4;  // each precision has its own order of sums (see k_jac_record)
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const bool live = k < nnzb;
   Rates r = rin;
@@ -724,22 +750,33 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
     const int32_t e = inc[inc_ptr[k]];
     r = rates_at(rin, tri[3 * (int64_t)(e / 9) + (e % 9) / 3]);
   }
-  // sums over the block's triangles, started from the first one (an FP64 add costs as much
-  // as a product): a block is on the diagonal in all of its triangles or in none, so the
-  // mass weight multiplies once
   T M = 0, Mr = 0, K = 0, G[4] = {0, 0, 0, 0}, P[4] = {0, 0, 0, 0};
-  if (live) {
-    const int32_t q0 = inc_ptr[k], q1 = inc_ptr[k + 1];
-    auto entry = [&](int32_t e, const T*& R, const T*& g, const T*& pm, int& s) {
-      const int32_t t = e / 9, ab = e - 9 * t;
-      const int a = ab / 3, b = ab - 3 * a;
-      s = sym(a, b);
-      R = rec + (int64_t)REC * t;
-      g = R + REC_G + 4 * a;
-      pm = R + REC_P + 4 * s;
-    };
-    const T *R, *g, *pm;
-    int s;
+  auto entry = [&](int32_t e, const T*& R, const T*& g, const T*& pm, int& s) {
+    const int32_t t = e / 9, ab = e - 9 * t;
+    const int a = ab / 3, b = ab - 3 * a;
+    s = sym(a, b);
+    R = rec + (int64_t)REC * t;
+    g = R + REC_G + 4 * a;
+    pm = R + REC_P + 4 * s;
+  };
+  const T *R, *g, *pm;
+  int s;
+  const int32_t q0 = live ? inc_ptr[k] : 0, q1 = live ? inc_ptr[k + 1] : 0;
+  if constexpr (F32) {
+    for (int32_t q = q0; q < q1; ++q) {
+      entry(inc[q], R, g, pm, s);
+      M += R[0] * (s < 3 ? T(2.0 / 12.0) : T(1.0 / 12.0));
+      if (RULE == 1 && s < 3) Mr += R[0] * T(1.0 / 3.0);
+      K += R[REC_K + s];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (!PIC) G[c] += g[c];
+        P[c] += pm[c];
+      }
+    }
+  } else if (live) {
+    // started from the first triangle (an FP64 add costs as much as a product): a block is on
+    // the diagonal in all of its triangles or in none, so the mass weight multiplies once
     entry(inc[q0], R, g, pm, s);
     const bool diag = s < 3;
     T area = R[0];
@@ -764,14 +801,14 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
   }
   if (RULE == 0) Mr = M;
   // K, G and P arrive scaled by dt (G_c by dt nubar_c), see k_jac_record
-  T rk[13];
+  T rk[11];
   rate_consts<T>(rin, r, rk);
   const T dt = rk[0];
   const T nu0 = rk[1], nu1 = rk[2], nu2 = rk[3], nu3 = rk[4];
   const T dMr = dt * Mr;
-  const T alpha = rk[5], mu = rk[6], sigma = rk[7], ge = rk[8], gr = rk[9], gd = rk[10], outE = rk[11], outI = rk[12];
-  // both zero in the paper's runs: no FP64 products then
-  const bool births = sizeof(T) == 4 || alpha != T(0), deaths = sizeof(T) == 4 || mu != T(0);
+  const T alpha = rk[5], mu = rk[6], sigma = rk[7], ge = rk[8], gr = rk[9], gd = rk[10];
+  // FP64: births and deaths are both zero in the paper's runs, no products then
+  const bool births = alpha != T(0), deaths = mu != T(0);
   T B[5][5];
 #pragma unroll
   for (int i = 0; i < 5; ++i)
@@ -788,8 +825,8 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
     B[1][1] = M + nu1 * K - P[2] + (sigma + ge + mu) * dMr;
   } else {
     // rows S, E: transmission derivative row  dT/du_c' = P0 + [S]P1 + [E]P2 + [I]P3
-    T rS = G[0] + P[0];
-    if (births) rS -= alpha * dMr;
+    T rS = F32 ? G[0] - alpha * dMr + P[0] : G[0] + P[0];
+    if (!F32 && births) rS -= alpha * dMr;
     const T rE = G[1] - P[0];
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
@@ -798,22 +835,32 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
       B[2][c] = G[2];
       B[3][c] = G[3];
     }
-    T dS = P[1] + fmaR(nu0, K, M);
-    if (deaths) dS += mu * dMr;
-    B[0][0] += dS;
+    if constexpr (F32) {
+      B[0][0] += M + nu0 * K + P[1] + mu * dMr;
+      B[1][1] += M + nu1 * K - P[2] + (sigma + ge + mu) * dMr;
+    } else {
+      T dS = P[1] + fma(nu0, K, M);
+      if (deaths) dS += mu * dMr;
+      B[0][0] += dS;
+      B[1][1] += fma(r.out_e, dMr, fma(nu1, K, M)) - P[2];
+    }
     B[0][1] += P[2];
     B[0][2] += P[3];
     B[1][0] -= P[1];
-    B[1][1] += fmaR(outE, dMr, fmaR(nu1, K, M)) - P[2];
     B[1][2] -= P[3];
   }
   B[2][1] -= sigma * dMr;
-  B[2][2] += fmaR(outI, dMr, fmaR(nu2, K, M));
   B[3][1] -= ge * dMr;
   B[3][2] -= gr * dMr;
-  T dR = fmaR(nu3, K, M);
-  if (deaths) dR += mu * dMr;
-  B[3][3] += dR;
+  if constexpr (F32) {
+    B[2][2] += M + nu2 * K + (gr + gd + mu) * dMr;
+    B[3][3] += M + nu3 * K + mu * dMr;
+  } else {
+    B[2][2] += fma(r.out_i, dMr, fma(nu2, K, M));
+    T dR = fma(nu3, K, M);
+    if (deaths) dR += mu * dMr;
+    B[3][3] += dR;
+  }
   B[4][2] -= gd * dMr;
   B[4][4] += M;
   stage_store25<T>(B, k, nnzb, val);

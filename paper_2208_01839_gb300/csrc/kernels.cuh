@@ -24,13 +24,6 @@ struct Rates {
     out_e = sigma + ge + mu;
     out_i = gr + gd + mu;
   }
-  // the FP32 kernels' copies: dt, nu, alpha, mu, sigma, ge, gr, gd, out_e, out_i, A, bi, be
-  float f[16];
-  void floats() {
-    const double v[16] = {dt,    nu[0], nu[1], nu[2], nu[3], alpha, mu, sigma,
-                          ge,    gr,    gd,    out_e, out_i, A,     bi, be};
-    for (int i = 0; i < 16; ++i) f[i] = (float)v[i];
-  }
   // ensembles: per-sample rows [A, bi, be, sigma, ge, gr, gd, alpha, mu, nu0..3] of a
   // device table, sample = internal node / nper (NULL: the scalars above for every node)
   const double* tab;

@@ -144,7 +144,6 @@ Rates make_rates(const seird_ctx* ctx) {
   for (int c = 0; c < 4; ++c) r.nu[c] = p.nu[c];
   r.dt = ctx->opt.dt;
   r.sums();
-  r.floats();
   return r;
 }
 
