@@ -613,8 +613,9 @@ int norm2(seird_ctx* ctx, const double* x, double* out) {
 bool verbose();
 
 // Launch-shape autotuner (options.autotune): times the candidates on the context's own
-// vectors (V[0] holds the first Krylov vector; the Gram-Schmidt candidates run at depth 8
-// with V[1..7] set to copies of it, which GMRES overwrites later) and keeps the fastest.
+// vectors (V[0] holds the first Krylov vector; the Gram-Schmidt candidates run at depth 8, or
+// at the gmres_restart + 1 vectors there are, with V[1..] set to copies of it, which GMRES
+// overwrites later) and keeps the fastest.
 int autotune(seird_ctx* ctx) {
   ctx->tuned = true;
   const int64_t len = vlen(ctx);
@@ -646,7 +647,7 @@ int autotune(seird_ctx* ctx) {
       ctx->spmv_tb = tb;
     }
   }
-  const int nv = 8;
+  const int nv = std::min(8, ctx->opt.gmres_restart + 1);
   for (int k = 1; k < nv; ++k)
     CK(cudaMemcpyAsync(ctx->V + (int64_t)k * len, ctx->V, sizeof(double) * len, cudaMemcpyDeviceToDevice, s));
   CK(cudaMemcpyAsync(ctx->tune_buf, ctx->V, sizeof(double) * len, cudaMemcpyDeviceToDevice, s));
