@@ -63,3 +63,23 @@ def test_float32_values_are_widened_exactly():
         a, b = _spmv(rp, col, only, x), _spmv(rp, col, only.astype(np.float64), x)
         assert np.array_equal(a, b, equal_nan=True)
         assert np.array_equal(a, val[:, :, c].astype(np.float64).ravel(), equal_nan=True)
+
+
+def test_float32_special_values_are_widened_exactly():
+    """Zeros, the smallest and largest subnormals, the ends of every power of two (so of each
+    exponent), infinities and a NaN, in blocks of five rows of one value each."""
+    ends = np.arange(1, 255, dtype=np.uint32) << 23
+    bits = np.concatenate([[0, 1, 2, 0x3fffff, 0x400000, 0x7ffffe, 0x7fffff], ends, ends | 0x7fffff, ends | 0x2aaaaa,
+                           [0x7f800000, 0x7fc00000]]).astype(np.uint32)
+    val = np.concatenate([bits, bits | 0x80000000]).astype(np.uint32).view(np.float32)
+    assert len(val) == 1542 and (val == 0).sum() == 2 and np.isinf(val).sum() == 2 and np.isnan(val).sum() == 2
+    assert np.isin(np.float32([1e-45, 1.1754942e-38, 1.17549435e-38, 3.4028235e38, 1.0, -1.0, 2.0 ** 127]), val).all()
+    val = np.concatenate([val, np.zeros(-len(val) % 25, np.float32)]).reshape(-1, 5, 5)
+    rp = np.arange(len(val) + 1, dtype=np.int32)
+    col = np.zeros(len(val), dtype=np.int32)
+    for c in range(5):  # one column at a time: y holds the widened values themselves
+        only = np.zeros_like(val)
+        only[:, :, c] = val[:, :, c]
+        x = np.zeros(5)
+        x[c] = 1.0
+        assert np.array_equal(_spmv(rp, col, only, x), val[:, :, c].astype(np.float64).ravel(), equal_nan=True)
