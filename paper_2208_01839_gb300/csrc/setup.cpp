@@ -1010,6 +1010,31 @@ int64_t check_setup(const HostSetup& hs, std::string& first) {
       }
     }
   }
+  // ring placement: no stage overlaps one that need not have been consumed before it.  Rows of
+  // more blocks than the one-stage ring holds, up to SOLVE_RING_FULL, run with the longer ring
+  // only and are placed there all the same, though their stages exceed the check below.
+  for (int32_t q = 0; q < P && !bad; ++q) {
+    const int32_t f0 = hs.sp_fwd.sd_lev0[q], nF = hs.sp_fwd.sd_lev0[q + 1] - f0 - 1;
+    const int32_t l0 = hs.sp_bwd.sd_lev0[q], ng = nF + hs.sp_bwd.sd_lev0[q + 1] - l0 - 1;
+    auto rec = [&](int32_t g) { return g < nF ? hs.sp_fwd.stage[f0 + g] : hs.sp_bwd.stage[l0 + g - nF]; };
+    for (int v = 0; v < 2 && hs.max_row_blocks <= (v == 0 ? SOLVE_RING_FULL : SOLVE_RING_HALF); ++v)
+      for (int32_t g = 0, free_to = -1; g < ng && !bad; ++g) {  // stages up to free_to have been consumed
+        const int4 st = rec(g);
+        const int32_t dist = stage_distance(st, v), blocks = solve_ring_blocks(P, hs.fp32, v == 1, hs.max_row_blocks);
+        if (dist != SOLVE_FREE) free_to = std::max(free_to, g - dist);
+        fail(dist >= 1 && (dist <= SOLVE_SLOTS || dist == SOLVE_FREE) && g - free_to <= SOLVE_SLOTS, "stage slot reused");
+        fail(g != nF || free_to == g - 1, "backward sweep starts early");
+        const int32_t rb = stage_block_offset(st, v), rr = stage_row_offset(st, v);
+        fail(rb + stage_blocks(st) <= blocks + SOLVE_RING_SPARE && rr + stage_rows(st) <= solve_ring_rows(blocks),
+             "stage wraps around a ring");
+        for (int32_t o = std::max(0, free_to + 1); o < g; ++o) {
+          const int4 so = rec(o);
+          const int32_t ob = stage_block_offset(so, v), orr = stage_row_offset(so, v);
+          fail(rb >= ob + stage_blocks(so) || ob >= rb + stage_blocks(st), "stages overlap in the factor ring");
+          fail(rr >= orr + stage_rows(so) || orr >= rr + stage_rows(st), "stages overlap in the row ring");
+        }
+      }
+  }
   // solve plans: each stage fits the shared-memory rings, every dependency of a row
   // lies in an earlier stage, and the records number the entries by sweep position
   for (int dir = 0; dir < 2 && !bad; ++dir) {
@@ -1063,29 +1088,6 @@ int64_t check_setup(const HostSetup& hs, std::string& first) {
       }
       if (dir == 1) fail(owned == hs.own_ptr[q + 1] - hs.own_ptr[q], "owned rows written once");
     }
-  }
-  // ring placement: no stage overlaps one that need not have been consumed before it
-  for (int32_t q = 0; q < P && !bad && hs.max_row_blocks <= SOLVE_RING_HALF; ++q) {
-    const int32_t f0 = hs.sp_fwd.sd_lev0[q], nF = hs.sp_fwd.sd_lev0[q + 1] - f0 - 1;
-    const int32_t l0 = hs.sp_bwd.sd_lev0[q], ng = nF + hs.sp_bwd.sd_lev0[q + 1] - l0 - 1;
-    auto rec = [&](int32_t g) { return g < nF ? hs.sp_fwd.stage[f0 + g] : hs.sp_bwd.stage[l0 + g - nF]; };
-    for (int v = 0; v < 2; ++v)
-      for (int32_t g = 0, free_to = -1; g < ng && !bad; ++g) {  // stages up to free_to have been consumed
-        const int4 st = rec(g);
-        const int32_t dist = stage_distance(st, v), blocks = solve_ring_blocks(P, hs.fp32, v == 1, hs.max_row_blocks);
-        if (dist != SOLVE_FREE) free_to = std::max(free_to, g - dist);
-        fail(dist >= 1 && (dist <= SOLVE_SLOTS || dist == SOLVE_FREE) && g - free_to <= SOLVE_SLOTS, "stage slot reused");
-        fail(g != nF || free_to == g - 1, "backward sweep starts early");
-        const int32_t rb = stage_block_offset(st, v), rr = stage_row_offset(st, v);
-        fail(rb + stage_blocks(st) <= blocks + SOLVE_RING_SPARE && rr + stage_rows(st) <= solve_ring_rows(blocks),
-             "stage wraps around a ring");
-        for (int32_t o = std::max(0, free_to + 1); o < g; ++o) {
-          const int4 so = rec(o);
-          const int32_t ob = stage_block_offset(so, v), orr = stage_row_offset(so, v);
-          fail(rb >= ob + stage_blocks(so) || ob >= rb + stage_blocks(st), "stages overlap in the factor ring");
-          fail(rr >= orr + stage_rows(so) || orr >= rr + stage_rows(st), "stages overlap in the row ring");
-        }
-      }
   }
   // launch order: every subdomain once (each CTA writes only the nodes its subdomain
   // owns), longest first

@@ -1,8 +1,9 @@
 """The subdomain solve and factorisation where the small cases of test_gpu_solve_shapes do
 not reach: subdomains of thousands of rows whose dependencies leave the window of 256
-results that a CTA keeps in shared memory, in every ring; and rows longer than the 32
-blocks a warp holds in the 256-thread factorisation (more than 152 subdomains).  Against
-the oracle's block ILU sweeps, with its tolerances: 1e-10 in FP64, 1e-4 with FP32 factors."""
+results that a CTA keeps in shared memory, in every ring; rows longer than the 32 blocks a
+warp holds in the 256-thread factorisation (more than 152 subdomains); and rows of 119 to
+236 blocks, which a context takes with the longer ring only.  Against the oracle's block
+ILU sweeps, with its tolerances: 1e-10 in FP64, 1e-4 with FP32 factors."""
 import functools
 
 import numpy as np
@@ -115,6 +116,9 @@ def _wheel_apply(spokes, hub_last, count, fill, precision):
     with S.Solver(xy, tri, p, owner=owner, dt=0.5, overlap=0, ilu_fill=fill, precision=precision) as sv:
         sv.jacobian(U0)
         sv.precond_setup()
+        if spokes > 118:
+            with pytest.raises(S.SeirdError):
+                sv.set_launch_shapes(ilu_ring=118)
         got = sv.precond_apply(r.reshape(-1, 5)).ravel()
     return np.linalg.norm(got - ref) / np.linalg.norm(ref)
 
@@ -125,3 +129,34 @@ def _wheel_apply(spokes, hub_last, count, fill, precision):
 @pytest.mark.parametrize("spokes", [31, 32, 33, 100])
 def test_long_rows_in_the_256_thread_factorisation(spokes, count, precision):
     assert _wheel_apply(spokes, True, count, 1, precision) <= (1e-4 if precision else 1e-10)
+
+
+RING_COUNTS = [1, 153, 305, 457, 609]
+LONGEST = [(119, True), (187, True), (188, True), (189, True), (236, True), (119, False), (187, False), (188, False),
+           (235, False)]  # lower blocks, or upper ones besides the pivot: 236 blocks at most
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("count", RING_COUNTS)
+@pytest.mark.parametrize("spokes,hub_last", LONGEST)
+def test_placement_of_rows_beyond_the_one_stage_ring(spokes, hub_last, count, precision):
+    """The check reports such a stage only after it has found its place in the longer ring sound."""
+    xy, tri, owner = _wheel(spokes, hub_last, count)
+    with pytest.raises(S.SeirdError, match="stage exceeds the rings"):
+        S.setup_check(xy, tri, owner=owner, overlap=0, ilu_fill=0, precision=precision)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("count", RING_COUNTS)
+@pytest.mark.parametrize("spokes,hub_last", LONGEST)
+def test_rows_beyond_the_one_stage_ring(spokes, hub_last, count, precision):
+    assert _wheel_apply(spokes, hub_last, count, 0, precision) <= (1e-4 if precision else 1e-10)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("spokes,hub_last", [(237, True), (236, False)])
+def test_rows_beyond_the_longer_ring_are_refused(spokes, hub_last):
+    xy, tri, owner = _wheel(spokes, hub_last, 1)
+    with pytest.raises(S.SeirdError, match="more blocks than the solve's shared-memory ring"):
+        S.Solver(xy, tri, I.params_ontario(40.0), owner=owner, dt=0.5, overlap=0)
