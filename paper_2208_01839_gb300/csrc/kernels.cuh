@@ -32,17 +32,6 @@ struct Rates {
 constexpr int RATE_ROW = 13;
 
 #ifdef __CUDACC__
-// (double)f on the integer pipe: GB300 converts at its FP64 rate, so a conversion costs as much
-// as the FMA it feeds.  The exponent is rebiased (127 -> 1023) and the 23 fraction bits become
-// the leading ones of 52; subnormals, infinities and NaNs take the conversion instruction.
-__device__ __forceinline__ double widen(float f) {
-  const uint32_t b = __float_as_uint(f), m = b & 0x7fffffffu;
-  if (m - 0x00800000u >= 0x7f000000u && m != 0) return (double)f;
-  const uint32_t hi = m ? (m >> 3) + 0x38000000u : 0u;
-  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
-}
-__device__ __forceinline__ double widen(double d) { return d; }
-
 // The rates that hold at internal node `node` (its sample's row of the table).
 __device__ __forceinline__ Rates rates_at(const Rates& r, int64_t node) {
   if (!r.tab) return r;

@@ -14,8 +14,24 @@ namespace {
 
 constexpr int NVMAX = 65;  // restart <= 64 -> at most 65 basis vectors
 
-__device__ __forceinline__ double ld_val(const double* p) { return __ldg(p); }
-__device__ __forceinline__ double ld_val(const float* p) { return widen(__ldg(p)); }
+// (double)f on the integer pipe: GB300 converts at its FP64 rate, so a conversion costs as much
+// as the FMA it feeds.  The exponent is rebiased (127 -> 1023) and the 23 fraction bits become
+// the leading ones of 52; subnormals, infinities and NaNs take the conversion instruction.
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t b = __float_as_uint(f), m = b & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0) return (double)f;
+  const uint32_t hi = m ? (m >> 3) + 0x38000000u : 0u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+
+template <bool WIDEN>
+__device__ __forceinline__ double ld_val(const double* p) {
+  return __ldg(p);
+}
+template <bool WIDEN>
+__device__ __forceinline__ double ld_val(const float* p) {
+  return WIDEN ? widen(__ldg(p)) : (double)__ldg(p);
+}
 
 // y = A x (b == NULL) or y = b - A x, 5x5 blocks.  One thread per scalar output row (block
 // row i, row r): all 32 lanes of every warp do useful FP64 work, 25 FMA per block per 5 threads.
@@ -23,7 +39,10 @@ __device__ __forceinline__ double ld_val(const float* p) { return widen(__ldg(p)
 // rows differ in length it takes them longest first, each row's rank counted on the integer
 // pipe (rows of four to nine blocks, 1.95M blocks: 139.5 -> 102.8 us).  A mesh's rows are nearly
 // all alike; for the Jacobian the sort only costs (2.0M nodes: 595 -> 601 us).
-template <class VT, bool UNEVEN>
+// WIDEN (FP32 values of a caller's matrix): widened by shifts instead of converted.  300,007
+// rows of four to nine blocks 212 -> 202 us, 20,000 rows 27.5 -> 23.4; a mesh's Jacobian is
+// slower that way (250k nodes 167.8 -> 170.6) and converts.
+template <class VT, bool UNEVEN, bool WIDEN>
 __global__ void __launch_bounds__(512) k_bsr_spmv(int64_t nrow, const int32_t* __restrict__ rp,
                                                   const int32_t* __restrict__ col, const VT* __restrict__ val,
                                                   const double* __restrict__ x, const double* __restrict__ b,
@@ -64,11 +83,11 @@ __global__ void __launch_bounds__(512) k_bsr_spmv(int64_t nrow, const int32_t* _
     const int64_t j = __ldg(col + k);
     const VT* v = val + 25 * (int64_t)k + 5 * r;
     const double* xj = x + 5 * j;
-    acc = fma(ld_val(v + 0), __ldg(xj + 0), acc);
-    acc = fma(ld_val(v + 1), __ldg(xj + 1), acc);
-    acc = fma(ld_val(v + 2), __ldg(xj + 2), acc);
-    acc = fma(ld_val(v + 3), __ldg(xj + 3), acc);
-    acc = fma(ld_val(v + 4), __ldg(xj + 4), acc);
+    acc = fma(ld_val<WIDEN>(v + 0), __ldg(xj + 0), acc);
+    acc = fma(ld_val<WIDEN>(v + 1), __ldg(xj + 1), acc);
+    acc = fma(ld_val<WIDEN>(v + 2), __ldg(xj + 2), acc);
+    acc = fma(ld_val<WIDEN>(v + 3), __ldg(xj + 3), acc);
+    acc = fma(ld_val<WIDEN>(v + 4), __ldg(xj + 4), acc);
   }
   const int64_t g = 5 * i + r;
   y[g] = b ? b[g] - acc : acc;
@@ -460,7 +479,7 @@ template <class VT>
 void launch_spmv(int64_t nrow, const int32_t* rp, const int32_t* col, const VT* val, const double* x, double* y,
                  cudaStream_t s, int tb, const double* b) {
   if (nrow <= 0) return;
-  k_bsr_spmv<VT, false><<<(unsigned)((5 * nrow + tb - 1) / tb), tb, 0, s>>>(nrow, rp, col, val, x, b, y);
+  k_bsr_spmv<VT, false, false><<<(unsigned)((5 * nrow + tb - 1) / tb), tb, 0, s>>>(nrow, rp, col, val, x, b, y);
   count_launch();
 }
 template <class VT>
@@ -470,8 +489,11 @@ void launch_spmv_uneven(int64_t nrow, const int32_t* rp, const int32_t* col, con
   const int tb = 256, R = tb / 5;
   // up to one wave of CTAs the launch lasts as long as its longest row whatever their order
   // (a few thousand rows: 13.5 us plain, 14.3 sorted)
-  if (nrow <= 152 * 8 * (int64_t)R) return launch_spmv<VT>(nrow, rp, col, val, x, y, s, tb, nullptr);
-  k_bsr_spmv<VT, true><<<(unsigned)((nrow + R - 1) / R), tb, 0, s>>>(nrow, rp, col, val, x, nullptr, y);
+  constexpr bool W = sizeof(VT) == 4;
+  if (nrow <= 152 * 8 * (int64_t)R)
+    k_bsr_spmv<VT, false, W><<<(unsigned)((5 * nrow + tb - 1) / tb), tb, 0, s>>>(nrow, rp, col, val, x, nullptr, y);
+  else
+    k_bsr_spmv<VT, true, W><<<(unsigned)((nrow + R - 1) / R), tb, 0, s>>>(nrow, rp, col, val, x, nullptr, y);
   count_launch();
 }
 template void launch_spmv<double>(int64_t, const int32_t*, const int32_t*, const double*, const double*, double*,
