@@ -515,18 +515,23 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
     Tt.gy[a] = (T)Tg.gy[a];
     Tt.v[a] = Tg.v[a];
   }
-  T u[3][5], Nv[3], Nsum = T(0);
+  T u[3][5], Nv[3], Nbar = T(0);
+  auto densities = [&] {
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
+    for (int a = 0; a < 3; ++a) Nv[a] = u[a][0] + u[a][1] + u[a][2] + u[a][3] + u[a][4];
+  };
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
       u[a][c] = (T)U[5 * (int64_t)Tt.v[a] + c];
-      if (F32) Nsum += u[a][c];
+      if (F32) Nbar += u[a][c];
     }
-    Nv[a] = u[a][0] + u[a][1] + u[a][2] + u[a][3] + u[a][4];
+  if (!F32) {
+    densities();
+    Nbar = Nv[0] + Nv[1] + Nv[2];
   }
-  if (!F32) Nsum = Nv[0] + Nv[1] + Nv[2];
-  const T Nbar = Nsum * T(1.0 / 3.0);
+  Nbar *= T(1.0 / 3.0);
   T* out = rec + (int64_t)REC * t;
   out[0] = Tt.area;
   // N-weighted stiffness dt |T| mean(N) grad phi_a . grad phi_b
@@ -568,6 +573,7 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
 #pragma unroll
     for (int a = 0; a < 3; ++a) bv[a] = (T)bfield[Tt.v[a]];
   }
+  if (F32) densities();
   const T A = shr ? srk[0] : (T)r.A, bi = shr ? srk[1] : (T)r.bi, be = shr ? srk[2] : (T)r.be;
   auto infect = [&](T ksb, T (&rho)[NM]) {  // moments 2 and 3 from kappa s b
     rho[2] = F32 ? ksb * be : ksb;
@@ -674,12 +680,9 @@ __global__ void __launch_bounds__(128) k_jac_record(int64_t m, const int32_t* __
   }
   if (bad) atomicOr(err, 1);
 #pragma unroll
-  for (int s = 0; s < 6; ++s) {
-    out[REC_P + 4 * s] = P[0][s];
-    out[REC_P + 4 * s + 1] = P[1][s];
-    out[REC_P + 4 * s + 2] = F32 ? P[2][s] : be * P[2][s];
-    out[REC_P + 4 * s + 3] = F32 ? P[NM - 1][s] : bi * P[2][s];
-  }
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int s = 0; s < 6; ++s) out[REC_P + 4 * s + k] = F32 || k < 2 ? P[k < NM ? k : 0][s] : (k == 2 ? be : bi) * P[2][s];
   out[REC_K + 6] = T(0);
 }
 
@@ -737,10 +740,13 @@ __device__ __forceinline__ void stage_store25(const T (&B)[5][5], int64_t k, int
 // RULE: the reaction quadrature.  The degree-5 rule integrates the linear
 // reaction terms exactly (consistent mass Mr = M); the vertex rule lumps them
 // (Mr = |T|/3 on the diagonal pair only), and the Jacobian follows the residual.
+// outs: the rates out of E and I, sigma + gamma_E + mu and gamma_R + gamma_D + mu, summed on the
+// host for the FP64 form.  (As members of Rates they cost the FP32 gather 3 to 6%: 219,717
+// nodes, 71.8 -> 74.6 us with the degree-5 rule, 74.0 -> 78.8 with the vertex rule.)
 template <class T, bool PIC, int RULE>
 __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t* __restrict__ inc_ptr,
                                                     const int32_t* __restrict__ inc, const T* __restrict__ rec,
-                                                    const int32_t* __restrict__ tri, Rates rin,
+                                                    const int32_t* __restrict__ tri, Rates rin, double2 outs,
                                                     T* __restrict__ val) {
   constexpr bool F32 = sizeof(T) == 4;  // each precision has its own order of sums (see k_jac_record)
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -749,34 +755,40 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
   if (live && rin.tab) {  // the block row's node: row vertex of the first incident triangle
     const int32_t e = inc[inc_ptr[k]];
     r = rates_at(rin, tri[3 * (int64_t)(e / 9) + (e % 9) / 3]);
+    if (!F32) outs = make_double2(r.sigma + r.ge + r.mu, r.gr + r.gd + r.mu);
   }
   T M = 0, Mr = 0, K = 0, G[4] = {0, 0, 0, 0}, P[4] = {0, 0, 0, 0};
-  auto entry = [&](int32_t e, const T*& R, const T*& g, const T*& pm, int& s) {
-    const int32_t t = e / 9, ab = e - 9 * t;
-    const int a = ab / 3, b = ab - 3 * a;
-    s = sym(a, b);
-    R = rec + (int64_t)REC * t;
-    g = R + REC_G + 4 * a;
-    pm = R + REC_P + 4 * s;
-  };
-  const T *R, *g, *pm;
-  int s;
   const int32_t q0 = live ? inc_ptr[k] : 0, q1 = live ? inc_ptr[k + 1] : 0;
   if constexpr (F32) {
     for (int32_t q = q0; q < q1; ++q) {
-      entry(inc[q], R, g, pm, s);
-      M += R[0] * (s < 3 ? T(2.0 / 12.0) : T(1.0 / 12.0));
-      if (RULE == 1 && s < 3) Mr += R[0] * T(1.0 / 3.0);
+      const int32_t e = inc[q];
+      const int32_t t = e / 9, ab = e - 9 * t;
+      const int a = ab / 3, b = ab - 3 * a;
+      const T* R = rec + (int64_t)REC * t;
+      const int s = sym(a, b);
+      M += R[0] * (a == b ? T(2.0 / 12.0) : T(1.0 / 12.0));
+      if (RULE == 1 && a == b) Mr += R[0] * T(1.0 / 3.0);
       K += R[REC_K + s];
+      if (!PIC) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        if (!PIC) G[c] += g[c];
-        P[c] += pm[c];
+        for (int c = 0; c < 4; ++c) G[c] += R[REC_G + 4 * a + c];
       }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) P[c] += R[REC_P + 4 * s + c];
     }
   } else if (live) {
     // started from the first triangle (an FP64 add costs as much as a product): a block is on
     // the diagonal in all of its triangles or in none, so the mass weight multiplies once
+    auto entry = [&](int32_t e, const T*& R, const T*& g, const T*& pm, int& s) {
+      const int32_t t = e / 9, ab = e - 9 * t;
+      const int a = ab / 3, b = ab - 3 * a;
+      s = sym(a, b);
+      R = rec + (int64_t)REC * t;
+      g = R + REC_G + 4 * a;
+      pm = R + REC_P + 4 * s;
+    };
+    const T *R, *g, *pm;
+    int s;
     entry(inc[q0], R, g, pm, s);
     const bool diag = s < 3;
     T area = R[0];
@@ -842,7 +854,7 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
       T dS = P[1] + fma(nu0, K, M);
       if (deaths) dS += mu * dMr;
       B[0][0] += dS;
-      B[1][1] += fma(r.out_e, dMr, fma(nu1, K, M)) - P[2];
+      B[1][1] += fma(outs.x, dMr, fma(nu1, K, M)) - P[2];
     }
     B[0][1] += P[2];
     B[0][2] += P[3];
@@ -856,7 +868,7 @@ __global__ void __launch_bounds__(128) k_jac_gather(int64_t nnzb, const int32_t*
     B[2][2] += M + nu2 * K + (gr + gd + mu) * dMr;
     B[3][3] += M + nu3 * K + mu * dMr;
   } else {
-    B[2][2] += fma(r.out_i, dMr, fma(nu2, K, M));
+    B[2][2] += fma(outs.y, dMr, fma(nu2, K, M));
     T dR = fma(nu3, K, M);
     if (deaths) dR += mu * dMr;
     B[3][3] += dR;
@@ -1073,8 +1085,9 @@ static void jacobian_kernels(int64_t nnzb, int64_t m, const int32_t* tri, const 
     if (bfield) k_jac_record<1, true, T, PIC><<<g, tb, 0, s>>>(m, tri, xy, geo, U, bfield, r, rc, err);
     else k_jac_record<1, false, T, PIC><<<g, tb, 0, s>>>(m, tri, xy, geo, U, bfield, r, rc, err);
   }
-  if (rule == 0) k_jac_gather<T, PIC, 0><<<g2, tb, 0, s>>>(nnzb, inc_ptr, inc, rc, tri, r, val);
-  else k_jac_gather<T, PIC, 1><<<g2, tb, 0, s>>>(nnzb, inc_ptr, inc, rc, tri, r, val);
+  const double2 outs = make_double2(r.sigma + r.ge + r.mu, r.gr + r.gd + r.mu);
+  if (rule == 0) k_jac_gather<T, PIC, 0><<<g2, tb, 0, s>>>(nnzb, inc_ptr, inc, rc, tri, r, outs, val);
+  else k_jac_gather<T, PIC, 1><<<g2, tb, 0, s>>>(nnzb, inc_ptr, inc, rc, tri, r, outs, val);
 }
 
 void launch_jacobian(int64_t nnzb, int64_t m, const int32_t* tri, const double* xy, const double* geo, const double* U,
@@ -1215,7 +1228,6 @@ extern "C" int seird_residual_noalloc(int64_t n_nodes, int64_t n_tris, const dou
   r.mu = params->mu;
   for (int c = 0; c < 4; ++c) r.nu[c] = params->nu[c];
   r.dt = dt;
-  r.sums();
   launch_residual(n_nodes, n_tris, tri, xy, nullptr, u, u_prev, beta_field_dev, r, quadrature, nd, elem, inc_ptr, inc,
                   F, partial, nrm, err, s);
   e = cudaGetLastError();

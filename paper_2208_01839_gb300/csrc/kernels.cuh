@@ -16,14 +16,6 @@ struct Rates {
   double A, bi, be, sigma, ge, gr, gd, alpha, mu;
   double nu[4];
   double dt;
-  double out_e, out_i;  // sigma + gamma_E + mu, gamma_R + gamma_D + mu
-#ifdef __CUDACC__
-  __host__ __device__
-#endif
-  void sums() {
-    out_e = sigma + ge + mu;
-    out_i = gr + gd + mu;
-  }
   // ensembles: per-sample rows [A, bi, be, sigma, ge, gr, gd, alpha, mu, nu0..3] of a
   // device table, sample = internal node / nper (NULL: the scalars above for every node)
   const double* tab;
@@ -50,7 +42,6 @@ __device__ __forceinline__ Rates rates_at(const Rates& r, int64_t node) {
   q.nu[1] = t[10];
   q.nu[2] = t[11];
   q.nu[3] = t[12];
-  q.sums();
   return q;
 }
 #endif

@@ -143,7 +143,6 @@ Rates make_rates(const seird_ctx* ctx) {
   r.mu = p.mu;
   for (int c = 0; c < 4; ++c) r.nu[c] = p.nu[c];
   r.dt = ctx->opt.dt;
-  r.sums();
   return r;
 }
 
