@@ -150,9 +150,12 @@ __device__ __forceinline__ void reciprocals7(const double (&N)[7], double (&r)[7
   }
 }
 
-// Triangle t from the geometry table written at set-up (k_tri_geometry: |T|, the stiffness
-// |T| grad phi_a . grad phi_b of its three edges (0,1) (0,2) (1,2) and the gradients of the
-// hat functions, GEO doubles per triangle), or from the coordinates when there is no table.
+// Triangle t from the geometry tables written at set-up (k_tri_geometry), or from the
+// coordinates when there are none.  One table of |T| and the gradients of the hat functions
+// (8 doubles per triangle), and after its m triangles one of |T| and the stiffness
+// |T| grad phi_a . grad phi_b of the edges (0,1) (0,2) (1,2) (4 doubles): a reader takes whole
+// 32-byte sectors of one of them.  (In one table of ten doubles, 80 bytes apart, the FP32
+// record of 2.1M triangles took 475 us instead of 458.)
 __device__ __forceinline__ Tri tri_of(const int32_t* __restrict__ tri, const double* __restrict__ xy,
                                       const double* __restrict__ geo, int64_t t) {
   if (!geo) return load_tri(tri, xy, t);
@@ -160,15 +163,15 @@ __device__ __forceinline__ Tri tri_of(const int32_t* __restrict__ tri, const dou
   T.v[0] = tri[3 * t];
   T.v[1] = tri[3 * t + 1];
   T.v[2] = tri[3 * t + 2];
-  const double2* g = reinterpret_cast<const double2*>(geo + GEO * t);
-  const double2 g1 = g[2], g2 = g[3], g3 = g[4];
-  T.area = g[0].x;
-  T.gx[0] = g1.x;
-  T.gx[1] = g1.y;
-  T.gx[2] = g2.x;
-  T.gy[0] = g2.y;
-  T.gy[1] = g3.x;
-  T.gy[2] = g3.y;
+  const double2* g = reinterpret_cast<const double2*>(geo + 8 * t);
+  const double2 g0 = g[0], g1 = g[1], g2 = g[2], g3 = g[3];
+  T.area = g0.x;
+  T.gx[0] = g0.y;
+  T.gx[1] = g1.x;
+  T.gx[2] = g1.y;
+  T.gy[0] = g2.x;
+  T.gy[1] = g2.y;
+  T.gy[2] = g3.x;
   return T;
 }
 
@@ -184,7 +187,7 @@ struct TriEdges {
   int32_t v[3];
 };
 __device__ __forceinline__ TriEdges edges_of(const int32_t* __restrict__ tri, const double* __restrict__ xy,
-                                             const double* __restrict__ geo, int64_t t) {
+                                             const double* __restrict__ geo, int64_t m, int64_t t) {
   TriEdges E;
   if (!geo) {
     const Tri T = load_tri(tri, xy, t);
@@ -194,7 +197,7 @@ __device__ __forceinline__ TriEdges edges_of(const int32_t* __restrict__ tri, co
     for (int a = 0; a < 3; ++a) E.v[a] = T.v[a];
     return E;
   }
-  const double2* g = reinterpret_cast<const double2*>(geo + GEO * t);
+  const double2* g = reinterpret_cast<const double2*>(geo + 8 * m + 4 * t);
   const double2 g0 = g[0], g1 = g[1];
   E.area = g0.x;
   E.k[0] = g0.y;
@@ -212,12 +215,14 @@ __global__ void __launch_bounds__(256) k_tri_geometry(int64_t m, const int32_t* 
   const Tri T = load_tri(tri, xy, t);
   double k[3];
   edge_stiffness(T, k);
-  double2* g = reinterpret_cast<double2*>(geo + GEO * t);
-  g[0] = make_double2(T.area, k[0]);
-  g[1] = make_double2(k[1], k[2]);
-  g[2] = make_double2(T.gx[0], T.gx[1]);
-  g[3] = make_double2(T.gx[2], T.gy[0]);
-  g[4] = make_double2(T.gy[1], T.gy[2]);
+  double2* g = reinterpret_cast<double2*>(geo + 8 * t);
+  g[0] = make_double2(T.area, T.gx[0]);
+  g[1] = make_double2(T.gx[1], T.gx[2]);
+  g[2] = make_double2(T.gy[0], T.gy[1]);
+  g[3] = make_double2(T.gy[2], 0.0);
+  double2* e = reinterpret_cast<double2*>(geo + 8 * m + 4 * t);
+  e[0] = make_double2(T.area, k[0]);
+  e[1] = make_double2(k[1], k[2]);
 }
 
 // Node terms of the degree-5 residual, 8 doubles per node: w = u - u^n - dt L u (L the
@@ -263,7 +268,7 @@ __global__ void __launch_bounds__(128) k_residual_elem5(int64_t m, const int32_t
                                                         double* __restrict__ elem, int32_t* err) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= m) return;
-  const TriEdges T = edges_of(tri, xy, geo, t);
+  const TriEdges T = edges_of(tri, xy, geo, m, t);
   const Rates r = rates_at(rin, T.v[0]);
   double u[3][4], w[3][5], Nv[3], l[3], Fe[3][5];
 #pragma unroll

@@ -63,8 +63,8 @@ void set_global_error(const std::string& msg);
 cudaError_t upload_quadrature();  // quadrature tables to constant memory (checked, synchronised)
 
 // ---- launchers (defined in the .cu files) ----
-constexpr int GEO = 10;  // doubles per triangle of the geometry table
-// geo: per-triangle |T|, edge stiffness and hat-function gradients from launch_tri_geometry,
+constexpr int GEO = 12;  // doubles per triangle of the geometry tables
+// geo: per-triangle |T|, hat-function gradients and edge stiffness from launch_tri_geometry,
 // or NULL to compute them from xy; nd: 8 doubles per node of scratch (degree-5 rule)
 void launch_tri_geometry(int64_t m, const int32_t* tri, const double* xy, double* geo, cudaStream_t s);
 void launch_residual(int64_t n, int64_t m, const int32_t* tri, const double* xy, const double* geo, const double* U,
