@@ -44,12 +44,12 @@ FALLBACK_HBM_GBS = 6800.0
 # capture of each kernel class, as (bytes per launch there, units processed there,
 # seird_get_info key of those units); scaled to a launch by the units it processes
 # (traffic grows in proportion).  The SpMV was captured on the 200k-node case of the
-# same generator, the subdomain solve on 500k nodes in 111 subdomains, the size they
-# have at 18.4M nodes, with block ILU(2) factors in FP64 and ILU(3) in FP32.
+# same generator, the subdomain solve at full size (18.4M nodes, 4096 subdomains, block
+# ILU(2) factors in FP64 and ILU(3) in FP32, the default launch shapes).
 NCU_TRAFFIC = {
     ("spmv", "fp64"): (307.414e6, 1400635, "nnzb"),  # k_bsr_spmv<double>, 1.4M blocks
-    ("ilu_solve", "fp64"): (1687.524e6, 7125275, "subdomain_blocks"),  # k_ilu_solve<double, double, 7, 640, true>
-    ("ilu_solve", "mixed"): (1189.238e6, 9267025, "subdomain_blocks"),  # k_ilu_solve<float, float, 7, 640, true>
+    ("ilu_solve", "fp64"): (70.541e9, 264544907, "subdomain_blocks"),  # k_ilu_solve<double, double, 7, 188, false>
+    ("ilu_solve", "mixed"): (44.726e9, 344245751, "subdomain_blocks"),  # k_ilu_solve<float, float, 7, 236, false>
 }
 
 # kernel classes with one kernel launch per timed call
