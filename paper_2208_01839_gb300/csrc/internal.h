@@ -154,7 +154,7 @@ struct seird_ctx {
   int64_t n_per_sample = 0;
   double* rtab = nullptr;
   std::vector<int64_t> sample_tri_ptr;  // [n_samples+1] internal triangle range of each sample
-  // the coarse factorisation's fixed launch sequence (two launches per block
+  // the coarse factorisation's fixed launch sequence (one launch per block
   // column), captured once into a CUDA graph on a private stream and replayed
   cudaGraphExec_t coarse_graph = nullptr;
   int64_t coarse_graph_kernels = 0;

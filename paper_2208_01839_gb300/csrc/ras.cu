@@ -1,13 +1,14 @@
-// Restricted additive Schwarz preconditioner (Eq. RAS) with block-ILU(0)
+// Restricted additive Schwarz preconditioner (Eq. RAS) with block-ILU(k)
 // subdomain solves, and the coarse correction of Section 3.1 with the
 // per-subdomain, per-compartment constant coarse space Z:
 //   z = sum_p R_p^T D_p (L_p U_p)^{-1} R_p r  +  Z A_c^{-1} Z^T r,  A_c = Z^T J Z,
 // applied additively or, as in Eq. RAS_2L, multiplicatively (the J Z blocks
 // summed at set-up turn the second residual update into k_az_sub).
 // One CTA per subdomain for the factorization and the solves; rows of one
-// level of the ILU(0) dependency DAG are independent and run in parallel, with
-// a barrier between stages, and the solve numbers a subdomain's solution
-// entries by their position in the sweep.  The coarse matrix is block-banded
+// level of the factors' dependency DAG are independent and run in parallel, with
+// a barrier between stages.  The solve works on factors scaled by the inverted
+// pivots and numbers a subdomain's solution entries by their position in the
+// sweep.  The coarse matrix is block-banded
 // (subdomains in reverse Cuthill-McKee order) and factored by block LU with 5x5
 // pivot blocks inverted under partial pivoting, then inverted explicitly.
 #include <algorithm>
@@ -455,8 +456,8 @@ constexpr int SOLVE_DRAIN_POLLS = 1 << 20;
 // the stages in order and meet at a named barrier after each one (the rows of a level depend
 // on the rows of earlier levels), which the last of them joins when the next stage has
 // arrived, so that the others have no wait of their own; a stage's "empty" mbarrier then
-// completes.  (An mbarrier test takes 110 clocks, as long as a whole batch of FP32
-// products; a barrier of eight warps takes 28.)  Every wait is bounded; on a timeout the
+// completes.  (A test of a completed mbarrier takes 46 clocks, a barrier of eight warps
+// 28.)  Every wait is bounded; on a timeout the
 // kernel sets bit 3 of *err, lets every issued copy land and returns.
 // The work arrays y and z hold one padded row per sweep position.  The forward sweep leaves
 // its results in y, and in z at the row's backward position, where the backward sweep finds
