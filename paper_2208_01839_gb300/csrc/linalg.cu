@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(512) k_bsr_spmv(int64_t nrow, const int32_t* _
                                                   const int32_t* __restrict__ col, const VT* __restrict__ val,
                                                   const double* __restrict__ x, const double* __restrict__ b,
                                                   double* __restrict__ y) {
-  int64_t i;
+  int64_t i, g;  // block row and scalar row
   int r;
   if constexpr (UNEVEN) {
     __shared__ int32_t len[104];  // blockDim.x / 5 rows, at most 102
@@ -71,8 +71,9 @@ __global__ void __launch_bounds__(512) k_bsr_spmv(int64_t nrow, const int32_t* _
     }
     if (q >= nr) return;
     i = i0 + mine;
+    g = 5 * i + r;
   } else {
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (g >= 5 * nrow) return;
     i = g / 5;
     r = (int)(g - 5 * i);
@@ -89,7 +90,6 @@ __global__ void __launch_bounds__(512) k_bsr_spmv(int64_t nrow, const int32_t* _
     acc = fma(ld_val<WIDEN>(v + 3), __ldg(xj + 3), acc);
     acc = fma(ld_val<WIDEN>(v + 4), __ldg(xj + 4), acc);
   }
-  const int64_t g = 5 * i + r;
   y[g] = b ? b[g] - acc : acc;
 }
 
